@@ -424,11 +424,12 @@ hm_status hm_decompress_debug(hm_matrix* m, int32_t tier, int64_t u0, int64_t u1
  *   Errors: HM_ERR_ARG, HM_ERR_OOM, HM_ERR_CUDA, HM_ERR_UNSUPPORTED.
  * hm_lu_solve -- x := U^-1 L^-1 b for nrhs columns (device FP64, original
  *   point order, column-major, leading dimensions ldb, ldx >= n; x must not
- *   overlap b), stream-ordered, no sync.  Each column is one persistent
- *   cooperative launch: warps take the leaf solves (forward over the leaves,
- *   then backward) and the coefficient products t_b = S X^T z of the low-rank
- *   factor blocks in a dependency order, each waiting (bounded) for what it
- *   reads; values are decoded exactly (head + tail) and the arithmetic is FP64.
+ *   overlap b), stream-ordered, no sync.  Up to four columns share one persistent
+ *   cooperative launch: half of its blocks take the leaf solves (forward over the
+ *   leaves, then backward), the others the coefficient products t_b = S X^T z of
+ *   the low-rank factor blocks, in a dependency order, each waiting (bounded) for
+ *   what it reads; values are decoded exactly (head + tail) and the arithmetic is
+ *   FP64.  A column's result does not depend on nrhs.
  *   A wait that runs out latches HM_ERR_TIMEOUT (hm_lu_sync_status).
  *   Errors: HM_ERR_ARG, HM_ERR_STATE (not compressed), HM_ERR_CUDA.
  * hm_lu_sync_status -- as hm_sync_status, for the solve's error word.

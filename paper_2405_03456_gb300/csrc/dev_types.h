@@ -259,6 +259,36 @@ struct LuDep {
   int32_t flag, target;
 };
 
+// Schedule of the solve on the device (schedule_lu), derived from that list.  A
+// step is a row item; "need" counts the steps (in list order) that must be
+// finished before a value is final.  A step's columns are sorted by the moment
+// their multiplier becomes final; the last ones (at most LU_LATE, those that
+// need the step right before this one) are its late columns.
+constexpr int LU_LATE = 64;
+constexpr int LU_MAX_RHS = 4;    // right-hand sides of one launch
+struct alignas(16) LuSCol {      // a packed column: LuCol with its multiplier's dependency
+  uint64_t off;
+  double scale;
+  int32_t mult;                  // row (or coefficient, if flag >= 0) it multiplies; column items: its coefficient
+  int32_t need;                  // steps
+  int32_t flag, target;          // coefficient counter that must reach target (flag < 0: none)
+  uint16_t fb, em;
+  int32_t pad[3];
+};
+static_assert(sizeof(LuSCol) == 48, "LuSCol layout");
+struct LuStep {
+  int32_t r0, nr;                // the leaf's rows
+  int32_t e0, e1;                // early columns
+  int32_t l0, l1;                // late columns
+  int32_t t0;                    // diagonal triangle (nr columns)
+  int32_t need_rhs;              // backward: the step that gave the forward result of this leaf, + 1
+};
+struct LuCItem {                 // a column item: columns [c0, c0 + nc), nc <= 4
+  int32_t r0, nr, c0, nc;
+  int32_t flag;                  // counter it adds nc to
+  int32_t bwd;
+};
+
 enum { MODE_Y = 0, MODE_VEC = 1, MODE_VEC_ADD = 2 };
 enum { TIER_F32 = 0, TIER_FF = 1 };
 

@@ -13,10 +13,11 @@
 #include "program.h"
 
 namespace hm {
-cudaError_t launch_lusolve(int nsm, const LuCol* cols, const LuItem* items, int nitems, const LuDep* deps,
-                           const uint8_t* pay, const int32_t* perm, int n, const double* b, double* bz, double* w,
-                           double* xz, double* x, double* coef, int* flags, int nflags, int* err, cudaStream_t st);
-int lusolve_max_blocks();
+cudaError_t launch_lusolve(int nblk, int nr, const LuSCol* cols, const LuStep* steps, int nsteps, const LuCItem* citems,
+                           int ncitems, const int32_t* rowleaf, const int32_t* perm, int nl, int maxr,
+                           const uint8_t* pay, const double* b, int64_t ldb, double* x, int64_t ldx, double* w,
+                           double* xz, double* coef, int* ctl, int nflags, int* err, cudaStream_t st);
+int lusolve_max_blocks(int maxr);
 }  // namespace hm
 
 using namespace hm;
@@ -28,26 +29,28 @@ struct hm_lu {
   double eps = 0;
   int codec = 0, valr = 0;
   LuProgram prog;
-  int nsm = 0;
+  int nblk = 0;
   uint8_t* d_pay = nullptr;
-  LuCol* d_cols = nullptr;
-  LuItem* d_items = nullptr;
-  LuDep* d_deps = nullptr;
+  LuSCol* d_cols = nullptr;
+  LuStep* d_steps = nullptr;
+  LuCItem* d_citems = nullptr;
+  int32_t* d_rowleaf = nullptr;
   int32_t* d_perm = nullptr;
-  int* d_flags = nullptr;
+  int* d_ctl = nullptr;      // coefficient counters, frontier, claim counters, abort word
   int* d_err = nullptr;
-  double* d_coef = nullptr;
-  double* d_vec = nullptr;   // b, w, x in cluster order (3 n)
+  double* d_coef = nullptr;  // LU_MAX_RHS per coefficient
+  double* d_vec = nullptr;   // w, x in cluster order (LU_MAX_RHS per row)
   void release() {
-    for (void* p : {(void*)d_pay, (void*)d_cols, (void*)d_items, (void*)d_deps, (void*)d_perm, (void*)d_flags,
-                    (void*)d_err, (void*)d_coef, (void*)d_vec})
+    for (void* p : {(void*)d_pay, (void*)d_cols, (void*)d_steps, (void*)d_citems, (void*)d_rowleaf, (void*)d_perm,
+                    (void*)d_ctl, (void*)d_err, (void*)d_coef, (void*)d_vec})
       if (p) cudaFree(p);
     d_pay = nullptr;
     d_cols = nullptr;
-    d_items = nullptr;
-    d_deps = nullptr;
+    d_steps = nullptr;
+    d_citems = nullptr;
+    d_rowleaf = nullptr;
     d_perm = nullptr;
-    d_flags = nullptr;
+    d_ctl = nullptr;
     d_err = nullptr;
     d_coef = nullptr;
     d_vec = nullptr;
@@ -107,21 +110,20 @@ hm_status hm_lu_compress(hm_lu* F, double eps, int32_t codec, int32_t valr) {
     return HM_ERR_OOM;
   }
   if (!ok) return HM_ERR_UNSUPPORTED;
-  const int nb = lusolve_max_blocks();
-  if (nb <= 0) return HM_ERR_CUDA;
-  F->nsm = std::min(nb, nsm);
+  F->nblk = std::min(lusolve_max_blocks(F->prog.maxr), nsm);   // one block per SM
+  if (F->nblk < 2) return HM_ERR_CUDA;   // row blocks and column blocks
   const LuProgram& P = F->prog;
   std::vector<int32_t> perm((size_t)F->n);
   for (int64_t i = 0; i < F->n; ++i) perm[i] = (int32_t)F->L.ct.perm[i];
   cudaError_t e;
-  if ((e = up(&F->d_pay, P.pk.pay)) != cudaSuccess || (e = up(&F->d_cols, P.cols)) != cudaSuccess ||
-      (e = up(&F->d_items, P.items)) != cudaSuccess || (e = up(&F->d_deps, P.deps)) != cudaSuccess ||
-      (e = up(&F->d_perm, perm)) != cudaSuccess ||
-      (e = cudaMalloc(&F->d_flags, (size_t)(P.nflags + 2) * sizeof(int))) != cudaSuccess ||
+  if ((e = up(&F->d_pay, P.pk.pay)) != cudaSuccess || (e = up(&F->d_cols, P.scols)) != cudaSuccess ||
+      (e = up(&F->d_steps, P.steps)) != cudaSuccess || (e = up(&F->d_citems, P.citems)) != cudaSuccess ||
+      (e = up(&F->d_rowleaf, P.rowleaf)) != cudaSuccess || (e = up(&F->d_perm, perm)) != cudaSuccess ||
+      (e = cudaMalloc(&F->d_ctl, (size_t)(P.nflags + 4) * sizeof(int))) != cudaSuccess ||
       (e = cudaMalloc(&F->d_err, sizeof(int))) != cudaSuccess ||
       (e = cudaMemset(F->d_err, 0, sizeof(int))) != cudaSuccess ||
-      (e = cudaMalloc(&F->d_coef, (size_t)std::max<int64_t>(P.ncoef, 1) * sizeof(double))) != cudaSuccess ||
-      (e = cudaMalloc(&F->d_vec, (size_t)(3 * F->n) * sizeof(double))) != cudaSuccess) {
+      (e = cudaMalloc(&F->d_coef, (size_t)std::max<int64_t>(P.ncoef, 1) * LU_MAX_RHS * sizeof(double))) != cudaSuccess ||
+      (e = cudaMalloc(&F->d_vec, (size_t)(2 * F->n) * LU_MAX_RHS * sizeof(double))) != cudaSuccess) {
     F->release();
     return e == cudaErrorMemoryAllocation ? HM_ERR_OOM : HM_ERR_CUDA;
   }
@@ -141,10 +143,12 @@ hm_status hm_lu_solve(hm_lu* F, const double* b, int64_t ldb, double* x, int64_t
   if (!(be <= x || xe <= b)) return HM_ERR_ARG;
   cudaStream_t st = (cudaStream_t)stream;
   const LuProgram& P = F->prog;
-  for (int64_t r = 0; r < nrhs; ++r)
-    if (launch_lusolve(F->nsm, F->d_cols, F->d_items, (int)P.items.size(), F->d_deps, F->d_pay, F->d_perm, (int)n,
-                       b + r * ldb, F->d_vec, F->d_vec + n, F->d_vec + 2 * n, x + r * ldx, F->d_coef, F->d_flags,
-                       (int)P.nflags, F->d_err, st) != cudaSuccess)
+  // up to LU_MAX_RHS right-hand sides share one launch
+  for (int64_t r = 0; r < nrhs; r += LU_MAX_RHS)
+    if (launch_lusolve(F->nblk, (int)std::min<int64_t>(LU_MAX_RHS, nrhs - r), F->d_cols, F->d_steps,
+                       (int)P.steps.size(), F->d_citems, (int)P.citems.size(), F->d_rowleaf, F->d_perm, (int)P.nleaves,
+                       P.maxr, F->d_pay, b + r * ldb, ldb, x + r * ldx, ldx, F->d_vec, F->d_vec + n * LU_MAX_RHS,
+                       F->d_coef, F->d_ctl, (int)P.nflags, F->d_err, st) != cudaSuccess)
       return HM_ERR_CUDA;
   return HM_OK;
 }

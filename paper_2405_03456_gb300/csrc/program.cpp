@@ -1250,6 +1250,71 @@ bool seq_dependencies(const Program& P, size_t first, size_t last, std::vector<S
 // and a low-rank block W S X^T contributes W|_c t_b with t_b = S X^T w_s, formed
 // by the block's column items once every leaf of s is solved.  The backward
 // pass is the same with U, leaves in reverse order, the upper triangle U_cc.
+//
+// The device does not run the items one by one: schedule_lu derives the leaf
+// steps and column items of the persistent launch from the same list.  Row items
+// complete in list order there, so a dependency on a leaf is a number of steps.
+static void schedule_lu(LuProgram& P, int64_t n) {
+  const int32_t nl = (int32_t)P.nleaves;
+  P.rowleaf.assign((size_t)n, 0);
+  for (int32_t f = 0, i = 0; i < nl; ++f)   // forward row items, in leaf order
+    if (P.items[f].kind == LU_ROW_L) {
+      std::fill_n(P.rowleaf.begin() + P.items[f].r0, P.items[f].nr, i++);
+      P.maxr = std::max(P.maxr, P.items[f].nr);
+    }
+  auto scol = [&](int32_t j, int32_t need, int32_t flag, int32_t target) {
+    const LuCol& c = P.cols[j];
+    P.scols.push_back(LuSCol{c.off, c.scale, c.mult, need, flag, target, c.fb, c.em, {0, 0, 0}});
+  };
+  // coefficients: counter, its final value, steps needed
+  std::vector<int32_t> cflag(P.ncoef, -1), cneed(P.ncoef, 0), total(P.nflags, 0);
+  for (const LuItem& it : P.items) {
+    if (it.kind != LU_COL_L && it.kind != LU_COL_U) continue;
+    const bool fwd = it.kind == LU_COL_L;
+    const int32_t need = fwd ? P.rowleaf[it.r0 + it.nr - 1] + 1 : 2 * nl - P.rowleaf[it.r0];
+    P.citems.push_back(LuCItem{it.r0, it.nr, (int32_t)P.scols.size(), it.c1 - it.c0, it.flag, fwd ? 0 : 1});
+    for (int32_t j = it.c0; j < it.c1; ++j) {
+      scol(j, need, -1, 0);
+      cflag[P.cols[j].mult] = it.flag;
+      cneed[P.cols[j].mult] = need;
+    }
+    total[it.flag] += it.c1 - it.c0;
+  }
+  int32_t s = 0;
+  for (const LuItem& it : P.items) {
+    if (it.kind != LU_ROW_L && it.kind != LU_ROW_U) continue;
+    const bool fwd = it.kind == LU_ROW_L;
+    struct Ref {
+      int32_t j, need, flag;
+    };
+    std::vector<Ref> refs;
+    for (int32_t j = it.c0; j < it.c1; ++j) {
+      const LuCol& c = P.cols[j];
+      if (c.flags & LC_COEF)
+        refs.push_back(Ref{j, cneed[c.mult], cflag[c.mult]});
+      else
+        refs.push_back(Ref{j, fwd ? P.rowleaf[c.mult] + 1 : 2 * nl - P.rowleaf[c.mult], -1});
+    }
+    std::stable_sort(refs.begin(), refs.end(), [](const Ref& a, const Ref& b) {
+      return a.need != b.need ? a.need < b.need : (a.flag >= 0) < (b.flag >= 0);
+    });
+    LuStep S{};
+    S.r0 = it.r0;
+    S.nr = it.nr;
+    S.need_rhs = fwd ? 0 : P.rowleaf[it.r0] + 1;
+    size_t late = refs.size();
+    while (late > 0 && refs.size() - late < (size_t)LU_LATE && refs[late - 1].need >= s) --late;
+    S.e0 = (int32_t)P.scols.size();
+    S.e1 = S.l0 = S.e0 + (int32_t)late;
+    S.l1 = S.e0 + (int32_t)refs.size();
+    for (const Ref& r : refs) scol(r.j, r.need, r.flag, r.flag >= 0 ? total[r.flag] : 0);
+    S.t0 = (int32_t)P.scols.size();
+    for (int32_t j = 0; j < it.nr; ++j) scol(it.tri + j, 0, -1, 0);
+    P.steps.push_back(S);
+    ++s;
+  }
+}
+
 bool build_lu_program(const HostMatrix& Lf, const HostMatrix& Uf, int codec, double eps, int valr,
                       LuProgram& P) {
   P = LuProgram();
@@ -1389,6 +1454,7 @@ bool build_lu_program(const HostMatrix& Lf, const HostMatrix& Uf, int codec, dou
   P.pk.align(16);
   P.pk.pay.resize(P.pk.pay.size() + 256, 0);   // 8-code groups of a column's last rows read past its end
   if (P.pk.pay.size() >= (1ull << 40) || P.ncoef >= INT32_MAX || P.cols.size() >= (size_t)INT32_MAX) return false;
+  schedule_lu(P, Lf.n);
   return true;
 }
 

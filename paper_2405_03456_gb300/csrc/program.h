@@ -141,6 +141,12 @@ struct LuProgram {
   int64_t ncoef = 0;        // coefficients of the low-rank blocks of both factors
   int64_t nleaves = 0;
   int64_t bytes_fp64 = 0;   // FP64 bytes of the same factors
+  // the device's schedule of the same list (schedule_lu)
+  std::vector<LuSCol> scols;
+  std::vector<LuStep> steps;
+  std::vector<LuCItem> citems;
+  std::vector<int32_t> rowleaf;   // leaf index of each row
+  int maxr = 1;                   // rows of the largest leaf
 };
 bool build_lu_program(const HostMatrix& L, const HostMatrix& U, int codec, double eps, int valr, LuProgram& P);
 

@@ -86,8 +86,8 @@ __device__ __forceinline__ void dot2(float& s, float& c, float dh, float dl, flo
 }
 
 // ---------------------------------------------------------------- decoding
-// Value i of 4 consecutive B-byte codes held in B little-endian words, placed
-// at the top of a 32-bit (B <= 4) or 64-bit (B >= 5) window.
+// Value i of 4 consecutive B-byte codes held in B little-endian words: its top
+// 32 bits (B >= 5), or the code placed at the top of a 32-bit window.
 template <int B, int I>
 __device__ __forceinline__ uint32_t top32(const uint32_t (&w)[B]) {
   constexpr int o = I * B + B - 4;
@@ -102,54 +102,54 @@ __device__ __forceinline__ uint32_t top32(const uint32_t (&w)[B]) {
   }
 }
 
+// Its 8 (B - 4) bits below that 32-bit window (B >= 5), right-aligned.
 template <int B, int I>
-__device__ __forceinline__ uint64_t top64(const uint32_t (&w)[B]) {
-  constexpr int o = I * B + B - 8;
-  if constexpr (o < 0) {
-    uint64_t v = ((uint64_t)w[1] << 32) | w[0];
-    return v << (8 * (-o));
-  } else {
-    constexpr int wi = o >> 2, sh = (o & 3) * 8;
-    uint64_t v = ((uint64_t)w[wi + 1] << 32) | w[wi];
-    if constexpr (sh == 0) {
-      return v;
-    } else {
-      return (v >> sh) | ((uint64_t)w[wi + 2] << (64 - sh));
-    }
-  }
+__device__ __forceinline__ uint32_t low32(const uint32_t (&w)[B]) {
+  static_assert(B >= 5, "codes of at most 4 bytes fit the window");
+  constexpr int o = I * B, wi = o >> 2, sh = (o & 3) * 8, nb = 8 * (B - 4);
+  if constexpr (nb == 32)
+    return w[wi];
+  else if constexpr (sh + nb == 32)
+    return w[wi] >> sh;
+  else if constexpr (sh + nb < 32)
+    return (w[wi] >> sh) & ((1u << nb) - 1u);
+  else
+    return __funnelshift_r(w[wi], w[wi + 1], sh) & ((1u << nb) - 1u);
 }
 
-// FP64 bit pattern -> value.  hi = the top 24 significant bits (the mantissa
-// cut to FP32's 23 bits); TIER_FF: lo = the rest, exact when the pattern has at
-// most 48 significant bits (every FPX e11 code up to m = 44; the 52-bit
-// mantissa of a raw FP64 value keeps its lo part rounded to 24 bits);
-// TIER_F32: lo = 0 (the FP32 tier's stated approximation: within 2^-22 + 2^-24
-// relative).  Values below 2^-126 give hi = 0, and lo is dropped below 2^-74.
-template <int TIER>
-__device__ __forceinline__ void split_f64bits(uint64_t P, float& hi, float& lo) {
-  const uint32_t sgn = (uint32_t)(P >> 32) & 0x80000000u;
-  const int E = (int)((P >> 52) & 0x7ff);
-  const uint64_t M = P & ((1ull << 52) - 1);
-  const uint32_t hb = (E >= 897) ? (((uint32_t)(E - 896) << 23) | (uint32_t)(M >> 29)) : 0u;
-  hi = __uint_as_float(hb | sgn);
+// Integer -> FP32, exact for x < 2^23 (BITS <= 23: one logic operation and one
+// FP32 subtraction on the 2^23 bit pattern), else rounded to nearest.
+template <int BITS>
+__device__ __forceinline__ float uint_to_float(uint32_t x) {
+  if constexpr (BITS <= 23)
+    return __uint_as_float(x | 0x4B000000u) - 8388608.0f;
+  else
+    return __uint2float_rn(x);
+}
+
+// FP64 bit pattern given by its high word and the next `nb` bits -> value.
+// hi = the top 24 significant bits (the mantissa cut to FP32's 23 bits);
+// TIER_FF: lo = the rest, exact when the pattern has at most 48 significant bits
+// (every FPX e11 code up to m = 44; the 52-bit mantissa of a raw FP64 value
+// keeps its lo part rounded to 24 bits); TIER_F32: lo = 0 (the FP32 tier's
+// stated approximation: within 2^-22 + 2^-24 relative).  Values below 2^-126
+// give hi = 0, and lo is dropped below 2^-74.  32-bit words throughout: GB300 has
+// no 64-bit shifts, and a 64-bit integer conversion runs on the FP64 pipe.
+template <int TIER, int NB>
+__device__ __forceinline__ void split_f64bits(uint32_t hw, uint32_t low, float& hi, float& lo) {
+  const uint32_t sgn = hw & 0x80000000u;
+  const int E = (int)((hw >> 20) & 0x7ffu);
+  // E - 896 in the top 9 bits (the two top bits of E shifted out, 896 mod 512 = 384), 23 mantissa bits below
+  const uint32_t t = __funnelshift_l(low << (32 - NB), hw, 3) - 0xC0000000u;
+  hi = __uint_as_float((E >= 897 ? t : 0u) | sgn);
   lo = 0.0f;
   if constexpr (TIER == TIER_FF) {
     if (E >= 949) {
-      float l = __uint2float_rn((uint32_t)(M & ((1u << 29) - 1)));
-      l *= __uint_as_float((uint32_t)(E - 948) << 23);
+      const float l = uint_to_float<NB - 3>(low & ((1u << (NB - 3)) - 1u)) *
+                      __uint_as_float((uint32_t)(E - 948 + 32 - NB) << 23);
       lo = __uint_as_float(__float_as_uint(l) ^ sgn);
     }
   }
-}
-
-// AFLP difference s - 1 of s = 2^f (1 + mant 2^-m') as float-float d + err,
-// given s_h (FP32, exact: s with its mantissa cut to 23 bits): d = fl(s_h - 1)
-// and err = (s_h - d) - 1, the exact rounding error of that subtraction (the
-// Fast2Sum error term: s_h >= 2 > 1, so both operations are exact).  err is 0
-// unless f >= 24.
-__device__ __forceinline__ void aflp_sub1(float sh, float& d, float& err) {
-  d = sh - 1.0f;
-  err = (sh - d) - 1.0f;
 }
 
 // Decode 4 consecutive values of format (F, B).
@@ -195,18 +195,31 @@ __device__ __forceinline__ void decode4(const uint32_t (&w)[B], int e, int m, fl
         l[2 * k + 1] = __uint_as_float(__float_as_uint(err.y) ^ (t1 & 0x80000000u));
       }
     }
-  } else if constexpr (F == 2 && B == 4) {
-    // AFLP in 32 bits.  The code fills the word (m' = 31 - e): the head
-    // s_h = 2^f (1 + top 23 mantissa bits) is exact in FP32, the sh = 8 - e = m' - 23
-    // bits shifted out form the tail t 2^(f - m'), t < 2^sh (exact: t via the
-    // 2^23 bit pattern).  s - 1 = d + err + tail; err + tail is exact for f <= 46.
-    // The FP32 tier keeps d = fl(s_h - 1), the value with its mantissa cut to
-    // 23 bits and then rounded once (within 2^-22 + 2^-24 relative).  Values in pairs.
+  } else if constexpr (F == 2) {
+    // AFLP of 4 bytes and more (m' = 8 B - 1 - e > 23).  The top 32 bits of the code
+    // hold the sign, f and the first 31 - e mantissa bits, so the head
+    // s_h = 2^f (1 + top 23 mantissa bits) comes from them alone and is exact in
+    // FP32; the other m' - 23 bits (the sh = 8 - e shifted out, then the code's
+    // lower bytes) form the tail t 2^(f - m').  s - 1 = d + err + tail with
+    // d = fl(s_h - 1) and err = (s_h - d) - 1 the exact rounding error of that
+    // subtraction (Fast2Sum, s_h >= 2; 0 unless f >= 24); err + tail is exact for
+    // f <= 46 and m' <= 47 (a 7-byte tail of up to 31 bits is rounded to 24).
+    // The FP32 tier keeps d: the mantissa cut to 23 bits and then rounded once
+    // (within 2^-22 + 2^-24 relative).  Values in pairs.
+    constexpr int nb = 8 * (B - 4);
     const int sh = 8 - e;
     const uint32_t tmask = (1u << sh) - 1u, mexp = (uint32_t)m << 23;
+    const uint32_t t[4] = {top32<B, 0>(w), top32<B, 1>(w), top32<B, 2>(w), top32<B, 3>(w)};
+    uint32_t lw[4] = {0u, 0u, 0u, 0u};
+    if constexpr (TIER == TIER_FF && B > 4) {
+      lw[0] = low32<B, 0>(w);
+      lw[1] = low32<B, 1>(w);
+      lw[2] = low32<B, 2>(w);
+      lw[3] = low32<B, 3>(w);
+    }
 #pragma unroll
     for (int k = 0; k < 2; ++k) {
-      const uint32_t c0 = w[2 * k], c1 = w[2 * k + 1];
+      const uint32_t c0 = t[2 * k], c1 = t[2 * k + 1];
       const uint32_t s0 = ((c0 & 0x7fffffffu) >> sh) + (127u << 23), s1 = ((c1 & 0x7fffffffu) >> sh) + (127u << 23);
       const float2 sv = make_float2(__uint_as_float(s0), __uint_as_float(s1));
       const float2 d = __fadd2_rn(sv, make_float2(-1.0f, -1.0f));
@@ -214,9 +227,13 @@ __device__ __forceinline__ void decode4(const uint32_t (&w)[B], int e, int m, fl
       h[2 * k + 1] = __uint_as_float(__float_as_uint(d.y) ^ (c1 & 0x80000000u));
       if constexpr (TIER == TIER_FF) {
         const float2 err = __fadd2_rn(__ffma2_rn(d, make_float2(-1.0f, -1.0f), sv), make_float2(-1.0f, -1.0f));
-        const float2 tv = __fadd2_rn(make_float2(__uint_as_float((c0 & tmask) | 0x4B000000u),
-                                                 __uint_as_float((c1 & tmask) | 0x4B000000u)),
-                                     make_float2(-8388608.0f, -8388608.0f));
+        const uint32_t x0 = ((c0 & tmask) << nb) | lw[2 * k], x1 = ((c1 & tmask) << nb) | lw[2 * k + 1];
+        float2 tv;
+        if constexpr (B <= 6)   // at most 23 bits
+          tv = __fadd2_rn(make_float2(__uint_as_float(x0 | 0x4B000000u), __uint_as_float(x1 | 0x4B000000u)),
+                          make_float2(-8388608.0f, -8388608.0f));
+        else
+          tv = make_float2(__uint2float_rn(x0), __uint2float_rn(x1));
         const float2 sc = make_float2(__uint_as_float((s0 & 0x7f800000u) - mexp),
                                       __uint_as_float((s1 & 0x7f800000u) - mexp));
         const float2 lv = __ffma2_rn(tv, sc, err);
@@ -224,34 +241,12 @@ __device__ __forceinline__ void decode4(const uint32_t (&w)[B], int e, int m, fl
         l[2 * k + 1] = __uint_as_float(__float_as_uint(lv.y) ^ (c1 & 0x80000000u));
       }
     }
-  } else if constexpr (F == 2) {                           // AFLP with m' > 23, B >= 5
-    uint64_t c[4];
-    constexpr int rs = 64 - 8 * B;
-    c[0] = top64<B, 0>(w) >> rs;
-    c[1] = top64<B, 1>(w) >> rs;
-    c[2] = top64<B, 2>(w) >> rs;
-    c[3] = top64<B, 3>(w) >> rs;
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const uint32_t sg = (uint32_t)(c[i] >> (8 * B - 1)) << 31;
-      const uint32_t f = (uint32_t)(c[i] >> m) & ((1u << e) - 1u);
-      const uint64_t mant = c[i] & ((1ull << m) - 1ull);
-      const uint32_t hb = ((f + 127u) << 23) | (uint32_t)(mant >> (m - 23));
-      float d, err;
-      aflp_sub1(__uint_as_float(hb), d, err);
-      h[i] = __uint_as_float(__float_as_uint(d) ^ sg);
-      if constexpr (TIER == TIER_FF) {
-        const uint64_t ml = mant & ((1ull << (m - 23)) - 1ull);
-        const float lv = __ull2float_rn(ml) * __uint_as_float((uint32_t)(f + 127 - m) << 23) + err;
-        l[i] = __uint_as_float(__float_as_uint(lv) ^ sg);
-      }
-    }
   } else {                                                  // FPX e11 or raw FP64
-    constexpr uint64_t mask = (B == 8) ? ~0ull : (~0ull << (8 * (8 - B)));
-    split_f64bits<TIER>(top64<B, 0>(w) & mask, h[0], l[0]);
-    split_f64bits<TIER>(top64<B, 1>(w) & mask, h[1], l[1]);
-    split_f64bits<TIER>(top64<B, 2>(w) & mask, h[2], l[2]);
-    split_f64bits<TIER>(top64<B, 3>(w) & mask, h[3], l[3]);
+    constexpr int nb = 8 * (B - 4);
+    split_f64bits<TIER, nb>(top32<B, 0>(w), low32<B, 0>(w), h[0], l[0]);
+    split_f64bits<TIER, nb>(top32<B, 1>(w), low32<B, 1>(w), h[1], l[1]);
+    split_f64bits<TIER, nb>(top32<B, 2>(w), low32<B, 2>(w), h[2], l[2]);
+    split_f64bits<TIER, nb>(top32<B, 3>(w), low32<B, 3>(w), h[3], l[3]);
   }
 }
 
@@ -328,14 +323,17 @@ __device__ __forceinline__ void ff_add_f2(float2& hi, float2& lo, float2 s) {
 }
 
 // Dot2 (Ogita-Rump-Oishi) on pairs: (s, c) += d * v per component, with d and
-// v float-float (dh + dl, vh + vl): TwoProduct by FMA, TwoSum of Knuth.
-__device__ __forceinline__ void dot2_2(float2& s, float2& c, float2 dh, float2 dl, float2 vh, float2 vl) {
-  const float2 p = __fmul2_rn(dh, vh);
-  const float2 pe = __ffma2_rn(dh, vh, make_float2(-p.x, -p.y));
+// v float-float (dh + dl, vh + vl): TwoProduct by FMA, TwoSum of Knuth.  ndh is
+// -dh (once per decoded pair, whatever the number of right-hand sides): the
+// negated product np needs no negation inside a paired instruction.
+__device__ __forceinline__ float2 neg2(float2 a) { return make_float2(-a.x, -a.y); }
+__device__ __forceinline__ void dot2_2(float2& s, float2& c, float2 dh, float2 ndh, float2 dl, float2 vh, float2 vl) {
+  const float2 np = __fmul2_rn(ndh, vh);
+  const float2 pe = __ffma2_rn(dh, vh, np);
   const float2 tail = __ffma2_rn(dh, vl, __ffma2_rn(dl, vh, pe));
-  const float2 s1 = __fadd2_rn(s, p);
+  const float2 s1 = sub2(s, np);
   const float2 bp = sub2(s1, s);
-  const float2 e = __fadd2_rn(sub2(s, sub2(s1, bp)), sub2(p, bp));
+  const float2 e = sub2(sub2(s, sub2(s1, bp)), __fadd2_rn(np, bp));   // (s - (s1 - bp)) + (p - bp)
   s = s1;
   c = __fadd2_rn(c, __fadd2_rn(e, tail));
 }
@@ -355,15 +353,17 @@ __device__ __forceinline__ void ff_add_dot2(float2& hi, float2& lo, float2 s, fl
 // 8 consecutive codes of format (F, B) at shared address a -> 4 FP32 pairs
 // (FP32 tier: AFLP as +-(s - 1), FPX e8 exactly, e11 / raw cut to FP32; see
 // decode4 for what each class gives).
-template <int F, int B>
-__device__ __forceinline__ void decode8p(uint32_t a, int e, int m, float2 (&h2)[4]) {
-  uint32_t w[2 * B];
+template <int B>
+__device__ __forceinline__ void load8(uint32_t a, uint32_t (&w)[2 * B]) {
 #pragma unroll
   for (int i = 0; i < B; ++i) {
     const uint2 t = lds64(a + 8u * i);
     w[2 * i] = t.x;
     w[2 * i + 1] = t.y;
   }
+}
+template <int F, int B>
+__device__ __forceinline__ void decode8w(const uint32_t (&w)[2 * B], int e, int m, float2 (&h2)[4]) {
   uint32_t w0[B], w1[B];
 #pragma unroll
   for (int i = 0; i < B; ++i) {
@@ -402,6 +402,13 @@ __device__ __forceinline__ void decode8p(uint32_t a, int e, int m, float2 (&h2)[
     h2[2] = make_float2(h1[0], h1[1]);
     h2[3] = make_float2(h1[2], h1[3]);
   }
+}
+
+template <int F, int B>
+__device__ __forceinline__ void decode8p(uint32_t a, int e, int m, float2 (&h2)[4]) {
+  uint32_t w[2 * B];
+  load8<B>(a, w);
+  decode8w<F, B>(w, e, m, h2);
 }
 
 // ---------------------------------------------------------------- tensor-core helpers

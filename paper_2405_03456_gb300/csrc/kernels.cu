@@ -16,7 +16,7 @@
 #include <cstdint>
 #include <cuda_runtime.h>
 
-#include "decode.cuh"
+#include "stream.cuh"
 
 namespace hm {
 
@@ -27,174 +27,20 @@ constexpr int C_STAGE = C_MOFF + PIECE_MAX_COLS * 8 + 16;
 constexpr int C_INFO = 16;                          // per-stage record (range flags, split / part, multiplier parity)
 constexpr int SMEM_TAIL = 128;                      // lane over-reads past the last stage
 
-__device__ __forceinline__ uint32_t pad16u(uint32_t x) { return (x + 15u) & ~15u; }
-
-// After a bounded wait gave up: wait (bounded) for the copies still in flight
-// into this warp's stages [i, issued) so that none lands after the block exits.
-template <int NS>
-__device__ void drain(uint64_t* bars, int i, int issued, uint32_t it0 = 0) {
-  for (int j = i; j < issued; ++j) {
-    const uint32_t u = it0 + (uint32_t)j;
-    mbar_wait(&bars[u % NS], (u / NS) & 1u, 50u);
-  }
-}
-
-// Programmatic dependent launch: a kernel lets the next one in the stream start
-// at once (its blocks take SM resources as they free up and run their prologue),
-// and waits for the previous one (completed, memory visible) before it reads
-// anything that kernel wrote.  Both are no-ops for ordinary launches.
-__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-
 // ---------------------------------------------------------------- column dots (phase A)
-// (s, c) += (s2, c2) for Dot2 pairs (TwoSum of the leading parts).
-template <int TIER>
-__device__ __forceinline__ void pair_add(float& s, float& c, float s2, float c2) {
-  if constexpr (TIER == TIER_F32) {
-    s += s2;
-  } else {
-    float t, e;
-    two_sum(s, s2, t, e);
-    s = t;
-    c += c2 + e;
-  }
-}
-
-// One halving step of a reduce-scatter over lanes: C values per lane, the
-// lane keeps the upper half (if `up`) or the lower half and adds the partner's
-// (lane ^ mask) copy of it.
-template <int TIER, int C>
-__device__ __forceinline__ void rscatter_step(float (&p)[8], float (&pc)[8], bool up, int mask) {
-  constexpr int H = C / 2;
-#pragma unroll
-  for (int k = 0; k < H; ++k) {
-    const float send = up ? p[k] : p[k + H];
-    const float keep = up ? p[k + H] : p[k];
-    const float keepc = up ? pc[k + H] : pc[k];
-    const float got = __shfl_xor_sync(HM_FULL, send, mask);
-    float gotc = 0.f;
-    if constexpr (TIER == TIER_FF) gotc = __shfl_xor_sync(HM_FULL, up ? pc[k] : pc[k + H], mask);
-    p[k] = keep;
-    pc[k] = keepc;
-    pair_add<TIER>(p[k], pc[k], got, gotc);
-  }
-}
-
-// Reduce-scatter of 8 per-column partials over the L lanes q of a group (lane
-// bits 0 .. log2 L - 1): afterwards lane q holds in p[0 .. 8/L) the group's
-// totals of columns q * 8/L + k.  Fixed exchange pattern (deterministic).
-template <int TIER, int L>
-__device__ __forceinline__ void reduce_scatter8(float (&p)[8], float (&pc)[8], int q) {
-  if constexpr (L == 8) {
-    rscatter_step<TIER, 8>(p, pc, (q & 4) != 0, 4);
-    rscatter_step<TIER, 4>(p, pc, (q & 2) != 0, 2);
-    rscatter_step<TIER, 2>(p, pc, (q & 1) != 0, 1);
-  } else {
-    static_assert(L == 4, "lanes per column");
-    rscatter_step<TIER, 8>(p, pc, (q & 2) != 0, 2);
-    rscatter_step<TIER, 4>(p, pc, (q & 1) != 0, 1);
-  }
-}
-
-// One column-dot piece at shared address sa.  A column's <= 64 rows are
-// spread over LPC = 64 / RL lanes of RL rows each; the warp's NG = 32 / LPC
-// lane groups take the columns g, g + NG, ... (x rows in registers).  The
-// column loop is rolled: each step shifts the partials down one register, so
-// after 8 steps p[t] holds column g + NG t of this round; a round covers
-// 8 NG columns and ends with a reduce-scatter over the LPC lanes.
-template <int TIER, int F, int B, int RL>
-__device__ __forceinline__ void cs_piece(uint32_t sa, int R, int nc, int flags, const float (&xh)[RL],
-                                         const float (&xl)[RL], int lane, F2 alpha, F2* __restrict__ partial,
+// One column-dot piece at shared address sa: lanes (g, q) = (lane / 8, lane % 8)
+// take rows 8q .. 8q + 7 of the columns j0 + g + 4 t, t < 8, of a round of 32
+// columns (x rows in registers): in the FP32 tier two columns per turn
+// (independent decodes), products summed in FP32 pairs; in the float-float tier
+// one column, Dot2 on row pairs.  The lanes' partials are exchanged as they come
+// (a reduce-scatter tree over the 8 lanes), so that the loop is rolled: a round of
+// 8 unrolled steps for each of the decode classes in use did not fit the
+// instruction cache (1.8 of 6.3 stall cycles per instruction).  Steps past the
+// last column are skipped as a whole; a ragged step masks its results.
+template <int TIER, int F, int B>
+__device__ __forceinline__ void cs_piece(uint32_t sa, int R, int nc, int flags, const float (&xh)[RPL],
+                                         const float (&xl)[RPL], int lane, F2 alpha, F2* __restrict__ partial,
                                          float2* __restrict__ vout) {
-  constexpr int LPC = SEG_ROWS / RL, NG = 32 / LPC, KO = 8 / LPC;
-  const int g = lane / LPC, q = lane % LPC;
-  const uint32_t stride = (((uint32_t)R + 15u) & ~15u) * B;
-  const bool fin = (flags & ITEM_FINAL) != 0;
-  const uint32_t cm = sa + (uint32_t)sizeof(CPieceHdr);          // CColMeta[nc]
-  const uint32_t sc = cm + 8u * nc;                                // F2[nc] (final only)
-  const uint32_t cb = cm + (fin ? 16u : 8u) * nc + (uint32_t)(RL * q * B);
-  const bool rows_on = RL * q < R;
-  for (int j0 = 0; j0 < nc; j0 += 8 * NG) {
-    float p[8], pc[8];
-#pragma unroll
-    for (int t = 0; t < 8; ++t) {
-      p[t] = 0.f;
-      pc[t] = 0.f;
-    }
-#pragma unroll 1
-    for (int t = 0; t < 8; ++t) {
-      const int j = j0 + g + NG * t;
-      float a = 0.f, ac = 0.f;
-      if (j < nc && rows_on) {
-        int e = 0, m = 0;
-        if constexpr (F == 2) {
-          const uint32_t em = lds32(cm + 8u * j) & 0xffffu;
-          e = em & 0xff;
-          m = em >> 8;
-        }
-        float2 a2 = make_float2(0.f, 0.f), ac2 = make_float2(0.f, 0.f);
-#pragma unroll
-        for (int hb = 0; hb < RL / RPL; ++hb) {
-          float h[8], l[8];
-          decode8s<TIER, F, B>(cb + (uint32_t)j * stride + (uint32_t)(hb * RPL * B), e, m, h, l);
-#pragma unroll
-          for (int u = 0; u < 8; u += 2) {
-            if constexpr (TIER == TIER_F32) {
-              a = fmaf(h[u], xh[hb * RPL + u], a);
-              a = fmaf(h[u + 1], xh[hb * RPL + u + 1], a);
-            } else {
-              dot2_2(a2, ac2, make_float2(h[u], h[u + 1]), make_float2(l[u], l[u + 1]),
-                     make_float2(xh[hb * RPL + u], xh[hb * RPL + u + 1]),
-                     make_float2(xl[hb * RPL + u], xl[hb * RPL + u + 1]));
-            }
-          }
-        }
-        if constexpr (TIER == TIER_FF) {   // even + odd rows (TwoSum of the leading parts)
-          a = a2.x;
-          ac = ac2.x;
-          pair_add<TIER>(a, ac, a2.y, ac2.y);
-        }
-      }
-#pragma unroll
-      for (int k = 0; k < 7; ++k) {
-        p[k] = p[k + 1];
-        pc[k] = pc[k + 1];
-      }
-      p[7] = a;
-      pc[7] = ac;
-    }
-    reduce_scatter8<TIER, LPC>(p, pc, q);
-#pragma unroll
-    for (int k = 0; k < KO; ++k) {
-      const int j = j0 + g + NG * (q * KO + k);
-      if (j < nc) {
-        const float s = p[k], c = pc[k];
-        const float h = s + c;
-        FF v = {h, c - (h - s)};
-        const int32_t out = (int32_t)lds32(cm + 8u * j + 4u);
-        if (fin) {
-          const uint2 f = lds64(sc + 8u * j);
-          v = ff_mul(v, FF{__uint_as_float(f.x), __uint_as_float(f.y)});
-          if (flags & ITEM_ALPHA) v = ff_mul(v, FF{alpha.hi, alpha.lo});
-          vout[out] = make_float2(v.hi, v.lo);
-        } else {
-          partial[out] = F2{v.hi, v.lo};
-        }
-      }
-    }
-  }
-}
-
-// FP32-tier column-dot piece: lanes (g, q) = (lane / 8, lane % 8) take rows
-// 8q .. 8q+7 of the columns g, g + 4, ...; two columns per step (independent
-// decodes), products summed in FP32 pairs; the 4 steps of a round are unrolled
-// so that p[t] holds column g + 4t; a round of 32 columns ends with the
-// reduce-scatter over the 8 lanes.  Steps past the last column are skipped as a
-// whole; a ragged step masks its results.
-template <int F, int B>
-__device__ __forceinline__ void cs_piece_f32(uint32_t sa, int R, int nc, int flags, const float2 (&x2)[4], int lane,
-                                             F2 alpha, F2* __restrict__ partial, float2* __restrict__ vout) {
-  constexpr int NG = 4;
   const int g = lane >> 3, q = lane & 7;
   const uint32_t stride = (((uint32_t)R + 15u) & ~15u) * B;
   const bool fin = (flags & ITEM_FINAL) != 0;
@@ -202,45 +48,85 @@ __device__ __forceinline__ void cs_piece_f32(uint32_t sa, int R, int nc, int fla
   const uint32_t sc = cm + 8u * nc;                                // F2[nc] (final only)
   const uint32_t cb = cm + (fin ? 16u : 8u) * nc + (uint32_t)(RPL * q * B);
   const bool rows_on = RPL * q < R;
-  for (int j0 = 0; j0 < nc; j0 += 8 * NG) {
-    float p[8], pc[8];
+  for (int j0 = 0; j0 < nc; j0 += 32) {
+    float c0 = 0.f, c0c = 0.f, d0 = 0.f, d0c = 0.f;
+#pragma unroll (TIER == TIER_F32 ? 2 : 1)
+    for (int i = 0; i < 4; ++i) {   // steps 2 i, 2 i + 1
+      float r[2] = {0.f, 0.f}, rc[2] = {0.f, 0.f};
+      if (j0 + 8 * i < nc) {
+        if constexpr (TIER == TIER_F32) {
 #pragma unroll
-    for (int t = 0; t < 8; ++t) {
-      p[t] = 0.f;
-      pc[t] = 0.f;
-    }
-    const int tmax = (nc - j0 + NG - 1) / NG;   // steps holding a column (same for the warp)
-#pragma unroll
-    for (int t = 0; t < 8; t += 2) {
-      float r[2] = {0.f, 0.f};
-      if (t < tmax) {
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          const int j = j0 + g + NG * (t + h);
-          const bool v = j < nc && rows_on;
-          const int jj = v ? j : 0;
-          int e = 0, m = 0;
-          if constexpr (F == 2) {
-            const uint32_t em = lds32(cm + 8u * jj) & 0xffffu;
-            e = em & 0xff;
-            m = em >> 8;
+          for (int h = 0; h < 2; ++h) {
+            const int j = j0 + g + 4 * (2 * i + h);
+            const bool v = j < nc && rows_on;
+            const int jj = v ? j : 0;
+            int e = 0, m = 0;
+            if constexpr (F == 2) {
+              const uint32_t em = lds32(cm + 8u * jj) & 0xffffu;
+              e = em & 0xff;
+              m = em >> 8;
+            }
+            float2 h2[4];
+            decode8p<F, B>(cb + (uint32_t)jj * stride, e, m, h2);
+            float2 a2 = __fmul2_rn(h2[0], make_float2(xh[0], xh[1]));
+            a2 = __ffma2_rn(h2[1], make_float2(xh[2], xh[3]), a2);
+            a2 = __ffma2_rn(h2[2], make_float2(xh[4], xh[5]), a2);
+            a2 = __ffma2_rn(h2[3], make_float2(xh[6], xh[7]), a2);
+            r[h] = v ? a2.x + a2.y : 0.f;
           }
-          float2 h2[4];
-          decode8p<F, B>(cb + (uint32_t)jj * stride, e, m, h2);
-          float2 a2 = __fmul2_rn(h2[0], x2[0]);
-          a2 = __ffma2_rn(h2[1], x2[1], a2);
-          a2 = __ffma2_rn(h2[2], x2[2], a2);
-          a2 = __ffma2_rn(h2[3], x2[3], a2);
-          r[h] = v ? a2.x + a2.y : 0.f;
+        } else {
+#pragma unroll 1
+          for (int h = 0; h < 2; ++h) {
+            const int j = j0 + g + 4 * (2 * i + h);
+            float a = 0.f, ac = 0.f;
+            if (j < nc && rows_on) {
+              int e = 0, m = 0;
+              if constexpr (F == 2) {
+                const uint32_t em = lds32(cm + 8u * j) & 0xffffu;
+                e = em & 0xff;
+                m = em >> 8;
+              }
+              float hv[8], lv[8];
+              decode8s<TIER, F, B>(cb + (uint32_t)j * stride, e, m, hv, lv);
+              float2 a2 = make_float2(0.f, 0.f), ac2 = make_float2(0.f, 0.f);
+#pragma unroll
+              for (int u = 0; u < 8; u += 2)
+                dot2_2(a2, ac2, make_float2(hv[u], hv[u + 1]), make_float2(-hv[u], -hv[u + 1]),
+                       make_float2(lv[u], lv[u + 1]), make_float2(xh[u], xh[u + 1]), make_float2(xl[u], xl[u + 1]));
+              a = a2.x;   // even + odd rows (TwoSum of the leading parts)
+              ac = ac2.x;
+              pair_add<TIER>(a, ac, a2.y, ac2.y);
+            }
+            r[0] = r[1];
+            rc[0] = rc[1];
+            r[1] = a;
+            rc[1] = ac;
+          }
         }
       }
-      p[t] = r[0];
-      p[t + 1] = r[1];
+      float p, pc;
+      exchange<TIER>(r[0], rc[0], r[1], rc[1], (q & 4) != 0, 4, p, pc);
+      if (i & 1) {
+        exchange<TIER>(c0, c0c, p, pc, (q & 2) != 0, 2, p, pc);
+        if (i == 1) {
+          d0 = p;
+          d0c = pc;
+          if (j0 + 16 >= nc) {   // the other half of the round holds no column
+            exchange<TIER>(d0, d0c, 0.f, 0.f, (q & 1) != 0, 1, d0, d0c);
+            break;
+          }
+        } else {
+          exchange<TIER>(d0, d0c, p, pc, (q & 1) != 0, 1, d0, d0c);
+        }
+      } else {
+        c0 = p;
+        c0c = pc;
+      }
     }
-    reduce_scatter8<TIER_F32, 8>(p, pc, q);
-    const int j = j0 + g + NG * q;
+    const int j = j0 + g + 4 * step_of_lane(q);
     if (j < nc) {
-      FF v = {p[0], 0.f};
+      const float h = d0 + d0c;
+      FF v = {h, d0c - (h - d0)};
       const int32_t out = (int32_t)lds32(cm + 8u * j + 4u);
       if (fin) {
         const uint2 f = lds64(sc + 8u * j);
@@ -342,26 +228,13 @@ __device__ __forceinline__ bool cs_range(const CsArgs& A, int p0, int n, uint8_t
       xv = hvin;
       xr = R;
     }
-    if constexpr (TIER == TIER_F32) {
-      const float2 x2[4] = {make_float2(xh[0], xh[1]), make_float2(xh[2], xh[3]), make_float2(xh[4], xh[5]),
-                            make_float2(xh[6], xh[7])};
-      switch (fb) {
+    switch (fb) {
 #define HM_CS(FF_, BB_) \
-  case ((FF_) << 4) | (BB_): cs_piece_f32<FF_, BB_>(sa, R, nc, (int)flags, x2, lane, A.alpha, A.partial, A.vout); break;
-        HM_FORMATS(HM_CS)
+  case ((FF_) << 4) | (BB_): cs_piece<TIER, FF_, BB_>(sa, R, nc, (int)flags, xh, xl, lane, A.alpha, A.partial, A.vout); break;
+      HM_FORMATS(HM_CS)
 #undef HM_CS
-        default:
-          latch_error(A.err, 1);
-      }
-    } else {
-      switch (fb) {
-#define HM_CS(FF_, BB_) \
-  case ((FF_) << 4) | (BB_): cs_piece<TIER, FF_, BB_, RL>(sa, R, nc, (int)flags, xh, xl, lane, A.alpha, A.partial, A.vout); break;
-        HM_FORMATS(HM_CS)
-#undef HM_CS
-        default:
-          latch_error(A.err, 1);
-      }
+      default:
+        latch_error(A.err, 1);
     }
     __syncwarp();
     if (issued < n) issue(issued);
@@ -396,20 +269,6 @@ __global__ void __launch_bounds__(NW * 32, 1)
 }
 
 // ---------------------------------------------------------------- row chunks (phase C)
-// Lane split of a row-chunk piece: G = ceil(R / 8) lanes per column, S = 32 / G
-// column slots, lane = slot G + q.  The divisions by the runtime G go through a
-// table: slot = (lane * ceil(1024 / G)) >> 10 is exact for lane < 1024 / G,
-// which holds for lane < 32 and G <= 16.
-__constant__ uint16_t c_div1024[17] = {0,    1024, 512, 342, 256, 205, 171, 147, 128,
-                                       114,  103,  94,  86,  79,  74,  69,  64};
-__constant__ uint8_t c_slots[17] = {0, 32, 16, 10, 8, 6, 5, 4, 4, 3, 3, 2, 2, 2, 2, 2, 2};
-__device__ __forceinline__ void lane_split(int R, int lane, int& G, int& S, int& slot, int& q) {
-  G = (R + RPL - 1) / RPL;
-  S = c_slots[G];
-  slot = (lane * (int)c_div1024[G]) >> 10;
-  q = lane - slot * G;
-}
-
 // Sum of the piece's columns into this lane's 8 rows: lanes (slot, q) take
 // rows 8q .. 8q+7 of the columns slot, slot + S, ...; FP32 sums (or Dot2
 // pairs) per piece, folded into the float-float row sums (row pairs
@@ -481,127 +340,12 @@ __device__ __forceinline__ void rs_piece(uint32_t sa, const PieceHdr& H, uint32_
       const float2 vh2 = make_float2(vh, vh), vl2 = make_float2(vl, vl);
 #pragma unroll
       for (int k = 0; k < 4; ++k)
-        dot2_2(s2[k], c2[k], make_float2(h[2 * k], h[2 * k + 1]), make_float2(l[2 * k], l[2 * k + 1]), vh2, vl2);
+        dot2_2(s2[k], c2[k], make_float2(h[2 * k], h[2 * k + 1]), make_float2(-h[2 * k], -h[2 * k + 1]),
+               make_float2(l[2 * k], l[2 * k + 1]), vh2, vl2);
     }
 #pragma unroll
     for (int k = 0; k < 4; ++k) ff_add_dot2(ahi[k], alo[k], s2[k], c2[k]);
   }
-}
-
-// Float-float row sums of a lane (RL rows), passed by value to the emit path.
-template <int RL>
-struct AccR {
-  FF v[RL];
-};
-
-// Write the finished rows g0 .. g0 + nr - 1 of a chunk (nr <= RL; a lane's rows).
-// Every global load the rows need (y through perm, the old coefficients, the row
-// scales) is issued before the first store, so the lane waits for one round trip
-// instead of one per row.  Coefficient vectors stay in float-float arithmetic
-// (FP64 instructions are scarce on this GPU); y takes the FP64 sum hi + lo.
-template <int MODE, int RL>
-__device__ __forceinline__ void rs_store_rows(const AccR<RL>& acc, int g0, int nr, F2 alpha_ff, double beta,
-                                              double* __restrict__ y, const int32_t* __restrict__ perm,
-                                              float2* __restrict__ vout, const F2* __restrict__ rowscale,
-                                              bool calpha) {
-  if constexpr (MODE == MODE_Y) {
-    int o[RL];
-#pragma unroll
-    for (int u = 0; u < RL; ++u) o[u] = u < nr ? __ldg(perm + g0 + u) : 0;
-    double yo[RL];
-#pragma unroll
-    for (int u = 0; u < RL; ++u) yo[u] = (u < nr && beta != 0.0) ? y[o[u]] : 0.0;
-#pragma unroll
-    for (int u = 0; u < RL; ++u) {
-      if (u < nr) {
-        const double val = ff_to_d(acc.v[u]);
-        y[o[u]] = (beta == 0.0) ? val : fma(beta, yo[u], val);
-      }
-    }
-  } else {
-    float2 old[RL], sc[RL];
-#pragma unroll
-    for (int u = 0; u < RL; ++u) {
-      old[u] = (MODE == MODE_VEC_ADD && u < nr) ? __ldcg(vout + g0 + u) : make_float2(0.f, 0.f);
-      sc[u] = (rowscale && u < nr) ? __ldg(reinterpret_cast<const float2*>(rowscale + g0 + u)) : make_float2(1.f, 0.f);
-    }
-#pragma unroll
-    for (int u = 0; u < RL; ++u) {
-      if (u < nr) {
-        FF v = acc.v[u];
-        if constexpr (MODE == MODE_VEC_ADD) v = ff_add(v, FF{old[u].x, old[u].y});
-        if (rowscale) v = ff_mul(v, FF{sc[u].x, sc[u].y});
-        if (calpha) v = ff_mul(v, FF{alpha_ff.hi, alpha_ff.lo});
-        vout[g0 + u] = make_float2(v.hi, v.lo);
-      }
-    }
-  }
-}
-
-// End of a warp's part of a chunk (hflags: piece header flags, bit 16 set when
-// the chunk is shared by several warps): reduce the column slots (fixed order), then
-// emit the rows, directly or through the fix-up of a chunk shared by warps (the
-// last part to arrive sums all parts in part order, so the result does not
-// depend on which warp finishes last).
-// Out of line: it runs once per part and keeps the piece loop compact.
-template <int MODE, int RL>
-__device__ __noinline__ bool rs_emit(AccR<RL> acc, int row0, int R, int hflags, int split, int pidx, int lane,
-                                     F2 alpha_ff, double beta, double* __restrict__ y,
-                                     const int32_t* __restrict__ perm, float2* __restrict__ vout,
-                                     const F2* __restrict__ rowscale, F2* __restrict__ fix,
-                                     int32_t* __restrict__ fixcnt, const Split* __restrict__ splits) {
-  static_assert(RL == RPL, "lanes hold RPL rows");
-  int G, S, slot, q;
-  lane_split(R, lane, G, S, slot, q);
-  // pairwise tree over the S column slots (slot s takes s + off when s is a
-  // multiple of 2 off): log2 S shuffle rounds, all rows of a round in flight
-  for (int off = 1; off < S; off <<= 1) {
-    float hi[RL], lo[RL];
-#pragma unroll
-    for (int u = 0; u < RL; ++u) {
-      hi[u] = __shfl_down_sync(HM_FULL, acc.v[u].hi, off * G);
-      lo[u] = __shfl_down_sync(HM_FULL, acc.v[u].lo, off * G);
-    }
-    if ((slot & (2 * off - 1)) == 0 && slot + off < S) {
-#pragma unroll
-      for (int u = 0; u < RL; ++u) acc.v[u] = ff_add(acc.v[u], FF{hi[u], lo[u]});
-    }
-  }
-  const bool mine = lane < G;   // slot 0 lanes hold the chunk's rows RL q .. RL q + RL-1
-  const int nr = mine ? min(RL, R - RL * q) : 0;
-  const bool calpha = (hflags & PH_CALPHA) != 0;
-  if (!(hflags & 0x10000)) {   // not shared with other warps
-    if (nr > 0) rs_store_rows<MODE, RL>(acc, row0 + RL * q, nr, alpha_ff, beta, y, perm, vout, rowscale, calpha);
-    return true;
-  }
-  const Split sp = splits[split];
-  F2* mypart = fix + (size_t)(sp.slot0 + pidx) * CHUNK_ROWS + RL * q;   // split, pidx: from the piece's split / part word
-#pragma unroll
-  for (int u = 0; u < RL; ++u)
-    if (u < nr) mypart[u] = F2{acc.v[u].hi, acc.v[u].lo};
-  __syncwarp();   // the part's rows before lane 0's release
-  int last = 0;
-  if (lane == 0) last = atom_add_acq_rel(&fixcnt[split], 1) == sp.nparts - 1;
-  last = __shfl_sync(HM_FULL, last, 0);
-  if (!last) return false;
-  __syncwarp();   // lane 0's acquire before the lanes read the other parts
-  if (nr > 0) {
-#pragma unroll
-    for (int u = 0; u < RL; ++u) acc.v[u] = FF{0.f, 0.f};
-    const F2* base = fix + (size_t)sp.slot0 * CHUNK_ROWS + RL * q;
-    for (int k = 0; k < sp.nparts; ++k) {   // the rows of one part: independent loads, then the sums
-      float2 v[RL];
-#pragma unroll
-      for (int u = 0; u < RL; ++u)
-        v[u] = u < nr ? __ldcg(reinterpret_cast<const float2*>(base + (size_t)k * CHUNK_ROWS + u))
-                      : make_float2(0.f, 0.f);
-#pragma unroll
-      for (int u = 0; u < RL; ++u) acc.v[u] = ff_add(acc.v[u], FF{v[u].x, v[u].y});
-    }
-    rs_store_rows<MODE, RL>(acc, row0 + RL * q, nr, alpha_ff, beta, y, perm, vout, rowscale, calpha);
-  }
-  if (lane == 0) fixcnt[split] = 0;   // ready for the next product
-  return true;
 }
 
 // Arguments of the row-chunk products shared by every range of a launch.
@@ -1238,22 +982,6 @@ __global__ void k_decode_debug(const DbgTask* __restrict__ tasks, int64_t ntask,
 }
 
 // ---------------------------------------------------------------- launchers
-// Launch with programmatic stream serialization (see pdl_trigger / pdl_wait).
-template <typename... KArgs, typename... Args>
-cudaError_t launch_pdl(void (*k)(KArgs...), unsigned grid, unsigned block, size_t smem, cudaStream_t st,
-                       Args... args) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(grid);
-  cfg.blockDim = dim3(block);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, k, args...);
-}
 template <int NW, int NS>
 constexpr size_t cs_smem() {
   return (size_t)NW * NS * (A_STAGE + 8) + SMEM_TAIL;

@@ -58,6 +58,18 @@ cudaError_t launch_rgemv_ms(int mode, const PieceCopy* pieces, const int32_t* wb
                             const float* vec, double alpha, F2 alpha_ff, double beta, double* y, int64_t ldy, int r,
                             const int32_t* perm, float* vout, const F2* rowscale, F2* fix, int32_t* fixcnt,
                             const Split* splits, const int32_t* fan, int32_t fan_base, int* err, cudaStream_t st);
+cudaError_t batch_init();
+int batch_shape(int tier, int nv);
+cudaError_t launch_gather_b(int nv, const double* x, int64_t ldx, int r, const int32_t* perm, int n, float2* v,
+                            cudaStream_t st);
+cudaError_t launch_gsum_b(int nv, const GsumOut* outs, int nouts, const F2* pscale, const float2* partial, F2 alpha,
+                          float2* v, cudaStream_t st);
+cudaError_t launch_cdot_b(int tier, int nv, const ItemCopy* items, const int32_t* wbeg, int nw, const uint8_t* pay,
+                          const float2* vec, F2 alpha, float2* partial, float2* vout, int* err, cudaStream_t st);
+cudaError_t launch_rgemv_b(int tier, int nv, int mode, const PieceCopy* pieces, const int32_t* wbeg, int nw,
+                           const uint8_t* pay, float2* vec, F2 alpha_ff, double beta, double* y, int64_t ldy, int r,
+                           const int32_t* perm, const F2* rowscale, F2* fix, int64_t nfix, int32_t* fixcnt, int nsplit,
+                           const Split* splits, const int32_t* fan, int32_t fan_base, int* err, cudaStream_t st);
 cudaError_t launch_decode(const uint8_t* p, int64_t n, int B, int fmt, int e, int m, double vmin,
                           double* out, cudaStream_t st);
 cudaError_t launch_decode_debug(int tier, const DbgTask* tasks, int64_t ntask, const uint8_t* pay, float2* out,
@@ -116,7 +128,12 @@ struct hm_matrix {
   float* d_vmr = nullptr;      // multi-RHS vectors: nvec x RP (FP32 tier)
   float* d_pmr = nullptr;      // multi-RHS column-dot partials: npartial x RP
   F2* d_fixmr = nullptr;       // multi-RHS fix-up rows: nfix_mr x CHUNK_ROWS x RP
-  int32_t* d_fixcnt = nullptr; // arrival counters of those chunks (reset by the last part)
+  // batches of up to BATCH_MAX right-hand sides: interleaved vectors, partials,
+  // fix-up rows.  In the FP32 tier they are the panel's buffers (a batch and a
+  // panel never run at the same time), in the float-float tier their own.
+  float2 *d_vb = nullptr, *d_pb = nullptr;
+  F2* d_fb = nullptr;
+  int32_t* d_fixcnt = nullptr; // arrival counters of those chunks (reset by the last part), per batch column
   float2* d_vec = nullptr;     // vector workspace (x, coefficient vectors)
   F2* d_part = nullptr;        // column-dot partial sums (float-float)
   int* d_err = nullptr;        // latched device error word
@@ -210,6 +227,13 @@ struct hm_matrix {
     d_perm.release();
     if (d_fix) cudaFree(d_fix);
     if (d_fixcnt) cudaFree(d_fixcnt);
+    if (d_vb && !d_vmr) {
+      cudaFree(d_vb);
+      cudaFree(d_pb);
+      cudaFree(d_fb);
+    }
+    d_vb = d_pb = nullptr;
+    d_fb = nullptr;
     if (d_vmr) cudaFree(d_vmr);
     if (d_pmr) cudaFree(d_pmr);
     if (d_fixmr) cudaFree(d_fixmr);
@@ -245,6 +269,14 @@ hm_matrix* new_matrix() { return new hm_matrix(); }
 
 namespace {
 
+// Columns of one batch pass (the widest kernels of each tier).
+constexpr int BATCH_MAX = 8, BATCH_MAX_FF = 4;
+
+// Fix-up slots (CHUNK_ROWS entries) that serve both a panel and a batch.
+int64_t fixmr_slots(const Program& P) {
+  return std::max<int64_t>({P.nfix_mr * RP, P.nfix * BATCH_MAX, 1});
+}
+
 std::once_flag g_kinit;
 cudaError_t g_kinit_err = cudaSuccess;
 
@@ -253,6 +285,7 @@ hm_status upload(hm_matrix* M) {
   cudaError_t e;
   std::call_once(g_kinit, [] {
     g_kinit_err = kernels_init();
+    if (g_kinit_err == cudaSuccess) g_kinit_err = batch_init();
     if (g_kinit_err == cudaSuccess) g_kinit_err = mr_init();
     if (g_kinit_err == cudaSuccess) g_kinit_err = tc_init();
   });
@@ -292,7 +325,7 @@ hm_status upload(hm_matrix* M) {
     return cuda_status(e);
   if ((e = cudaMalloc(&M->d_fix, std::max<int64_t>(P.nfix, 1) * CHUNK_ROWS * sizeof(F2))) != cudaSuccess)
     return cuda_status(e);
-  const size_t ncnt = std::max<size_t>(P.splits.size(), 1) * sizeof(int32_t);
+  const size_t ncnt = std::max<size_t>(P.splits.size(), 1) * BATCH_MAX * sizeof(int32_t);
   if ((e = cudaMalloc(&M->d_fixcnt, ncnt)) != cudaSuccess) return cuda_status(e);
   if ((e = cudaMemset(M->d_fixcnt, 0, ncnt)) != cudaSuccess) return cuda_status(e);
   if (P.tier == TIER_F32) {   // multi-RHS workspace (panels of RP right-hand sides; no fan-out slots)
@@ -301,8 +334,18 @@ hm_status upload(hm_matrix* M) {
     if ((e = cudaMemset(M->d_vmr, 0, nv)) != cudaSuccess) return cuda_status(e);
     if ((e = cudaMalloc(&M->d_pmr, (size_t)std::max<int64_t>(P.npartial, 1) * RP * sizeof(float))) != cudaSuccess)
       return cuda_status(e);
-    if ((e = cudaMalloc(&M->d_fixmr, (size_t)std::max<int64_t>(P.nfix_mr, 1) * CHUNK_ROWS * RP * sizeof(F2))) !=
-        cudaSuccess)
+    if ((e = cudaMalloc(&M->d_fixmr, (size_t)fixmr_slots(P) * CHUNK_ROWS * sizeof(F2))) != cudaSuccess)
+      return cuda_status(e);
+    static_assert(BATCH_MAX * sizeof(float2) <= RP * sizeof(float), "a batch's vectors fit the panel's");
+    M->d_vb = reinterpret_cast<float2*>(M->d_vmr);
+    M->d_pb = reinterpret_cast<float2*>(M->d_pmr);
+    M->d_fb = M->d_fixmr;
+  } else {
+    const size_t row = BATCH_MAX_FF * sizeof(float2);
+    if ((e = cudaMalloc(&M->d_vb, (size_t)(std::max<int64_t>(P.fan_base, 1) + SEG_ROWS) * row)) != cudaSuccess ||
+        (e = cudaMemset(M->d_vb, 0, (size_t)(std::max<int64_t>(P.fan_base, 1) + SEG_ROWS) * row)) != cudaSuccess ||
+        (e = cudaMalloc(&M->d_pb, (size_t)std::max<int64_t>(P.npartial, 1) * row)) != cudaSuccess ||
+        (e = cudaMalloc(&M->d_fb, (size_t)std::max<int64_t>(P.nfix, 1) * CHUNK_ROWS * row)) != cudaSuccess)
       return cuda_status(e);
   }
   if ((e = cudaMalloc(&M->d_err, sizeof(int))) != cudaSuccess) return cuda_status(e);
@@ -622,21 +665,83 @@ static hm_status run_program_mr(hm_matrix* M, double alpha, const double* x, int
 static hm_status run_program(hm_matrix* M, double alpha, const double* x, double beta, double* y,
                              cudaStream_t st);
 
+// One pass over r <= nv columns with the batch kernels.
+static cudaError_t run_launch_b(hm_matrix* M, const Launch& L, int nv, double alpha, const double* x, int64_t ldx,
+                                double beta, double* y, int64_t ldy, int r, cudaStream_t st) {
+  Program& P = M->prog;
+  const F2 aff = split_ff(alpha);
+  const int cf = batch_shape(P.tier, nv);
+  if (cf < 0) return cudaErrorInvalidValue;
+  switch (L.kind) {
+    case Launch::GATHER:
+      return launch_gather_b(nv, x, ldx, r, M->d_perm.p, (int)L.n, M->d_vb, st);
+    case Launch::CDOT:
+      return launch_cdot_b(P.tier, nv, M->d_items.p, M->d_wbeg.p + L.woff[cf], L.nw[cf], M->d_pay.p, M->d_vb, aff,
+                           M->d_pb, M->d_vb, M->d_err, st);
+    case Launch::GSUM:
+      return launch_gsum_b(nv, M->d_gout.p + L.off, (int)L.n, M->d_pscale.p, M->d_pb, aff, M->d_vb, st);
+    case Launch::FANOUT:   // the row chunks gather each multiplier row from its coefficient
+      return cudaSuccess;
+    case Launch::RGEMV:
+      return launch_rgemv_b(P.tier, nv, L.mode, M->d_pieces.p + (size_t)cf * P.npieces, M->d_wbeg.p + L.woff[cf],
+                            L.nw[cf], M->d_pay.p, M->d_vb, aff, beta, y, ldy, r, M->d_perm.p,
+                            L.use_rowscale ? M->d_rowscale_ff.p : nullptr, M->d_fb, P.nfix, M->d_fixcnt,
+                            (int)P.splits.size(), M->d_splits.p, M->d_fan.p, (int32_t)P.fan_base, M->d_err, st);
+  }
+  return cudaErrorInvalidValue;
+}
+
+static hm_status run_program_b(hm_matrix* M, int nv, double alpha, const double* x, int64_t ldx, double beta, double* y,
+                               int64_t ldy, int r, cudaStream_t st) {
+  for (const Launch& L : M->prog.launches) {
+    hm_matrix::Rec rec{(int)L.kind, nullptr, nullptr, L.bytes};
+    if (M->prof) {
+      rec.e0 = M->take_event();
+      rec.e1 = M->take_event();
+      cudaEventRecord(rec.e0, st);
+    }
+    if (run_launch_b(M, L, nv, alpha, x, ldx, beta, y, ldy, r, st) != cudaSuccess) return HM_ERR_CUDA;
+    if (M->prof) {
+      cudaEventRecord(rec.e1, st);
+      M->recs.push_back(rec);
+    }
+  }
+  return HM_OK;
+}
+
+// Width of the pass that takes the next of `rem` columns (1: a single product).
+// FP32 tier, N = 131072, eps = 1e-6 (ms): 1 column 0.222, 2 0.364, 3 0.465 and 4
+// 0.478 (width 4), 6 .. 8 0.85 (width 8), 5 0.70 as 4 + 1 and 0.79 at width 8; before,
+// 0.22 a column.  Float-float, n = 32768, eps = 1e-8: 0.159, 0.281, 0.476 at width 4;
+// before, 0.174 a column.
+static int pass_width(int tier, int64_t rem) {
+  if (rem <= 1) return 1;
+  if (rem == 2) return 2;
+  return tier == TIER_FF || rem <= 5 ? 4 : 8;
+}
+
 // All right-hand sides: panels of RP through the multi-RHS kernels (FP32
-// tier), the rest (or everything in the float-float tier) as one single-RHS
-// product per right-hand side.  A panel reads the matrix once; it costs about
-// as much as MR_MIN_RHS single products on GB300, so smaller remainders run
-// as single products.
+// tier), the rest (or everything in the float-float tier) in batch passes.  A
+// panel reads the matrix once, but costs more than a batch pass, so remainders
+// below MR_MIN_RHS run as batches.
 constexpr int64_t MR_MIN_RHS = 9;
 static hm_status run_all(hm_matrix* M, double alpha, const double* x, int64_t ldx, double beta, double* y,
                          int64_t ldy, int64_t nrhs, cudaStream_t st) {
   hm_status s = HM_OK;
   int64_t r0 = 0;
-  if (M->d_vmr)   // panels of RP; a panel of fewer than MR_MIN_RHS is cheaper as single products
+  if (M->d_vmr)   // panels of RP; a panel of fewer than MR_MIN_RHS is cheaper as batches
     for (; r0 < nrhs && nrhs - r0 >= MR_MIN_RHS && s == HM_OK; r0 += RP)
       s = run_program_mr(M, alpha, x + r0 * ldx, ldx, beta, y + r0 * ldy, ldy, (int)std::min<int64_t>(RP, nrhs - r0),
                          st);
-  for (int64_t r = r0; r < nrhs && s == HM_OK; ++r) s = run_program(M, alpha, x + r * ldx, beta, y + r * ldy, st);
+  while (r0 < nrhs && s == HM_OK) {
+    const int nv = pass_width(M->prog.tier, nrhs - r0);
+    const int r = (int)std::min<int64_t>(nv, nrhs - r0);
+    if (nv == 1)
+      s = run_program(M, alpha, x + r0 * ldx, beta, y + r0 * ldy, st);
+    else
+      s = run_program_b(M, nv, alpha, x + r0 * ldx, ldx, beta, y + r0 * ldy, ldy, r, st);
+    r0 += r;
+  }
   return s;
 }
 
@@ -1101,7 +1206,9 @@ hm_status hm_info(const hm_matrix* M, hm_info_t* o) {
                   H.n * 4;
   o->bytes_workspace = P.nvec * 8 + P.npartial * 8 + P.nfix * CHUNK_ROWS * 8;
   if (M->d_vmr)
-    o->bytes_workspace += ((P.fan_base + SEG_ROWS) + P.npartial) * RP * 4 + P.nfix_mr * CHUNK_ROWS * RP * 8;
+    o->bytes_workspace += ((P.fan_base + SEG_ROWS) + P.npartial) * RP * 4 + fixmr_slots(P) * CHUNK_ROWS * 8;
+  else if (M->d_vb)
+    o->bytes_workspace += ((P.fan_base + SEG_ROWS) + P.npartial + P.nfix * CHUNK_ROWS) * BATCH_MAX_FF * 8;
   o->nlaunches = (int64_t)P.launches.size();
   o->tier = P.tier;
   o->nunits = (int64_t)P.items.size() + P.npieces;

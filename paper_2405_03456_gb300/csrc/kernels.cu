@@ -710,9 +710,11 @@ __global__ void k_gsum(const GsumOut* __restrict__ outs, int nouts, const F2* __
 __global__ void k_gather(const double* __restrict__ x, const int32_t* __restrict__ perm, int n,
                          float2* __restrict__ xo) {
   pdl_trigger();
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  const int p = i < n ? __ldg(perm + i) : 0;
+  pdl_wait();   // x may be the previous kernel's result, and that kernel may still read xo
   if (i >= n) return;
-  FF f = ff_from_d(x[perm[i]]);
+  const FF f = ff_from_d(x[p]);
   xo[i] = make_float2(f.hi, f.lo);
 }
 
@@ -1121,8 +1123,7 @@ cudaError_t kernels_init() {
 
 cudaError_t launch_gather(const double* x, const int32_t* perm, int n, float2* xo, cudaStream_t st) {
   if (n <= 0) return cudaSuccess;
-  k_gather<<<(n + 255) / 256, 256, 0, st>>>(x, perm, n, xo);
-  return cudaGetLastError();
+  return launch_pdl(k_gather, (unsigned)((n + 255) / 256), 256, 0, st, x, perm, n, xo);
 }
 
 template <int NW, int NS>

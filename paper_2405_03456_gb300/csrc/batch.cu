@@ -52,54 +52,57 @@ __global__ void k_gather_b(const double* __restrict__ x, int64_t ldx, int r, con
   v[t] = make_float2(f.hi, f.lo);
 }
 
-// As the single product's segment sums: four lanes per output, lane k the
-// partials p0 + k, p0 + k + 4, ..., a fixed xor tree over the lanes.
+// As the single product's segment sums -- partials p0 + k, p0 + k + 4, ... by lane
+// group k, a fixed xor tree over the four groups -- with NV / 2 lanes per group,
+// two right-hand sides (16 bytes) each: a lane has no more sums in flight than
+// two, so that as many threads are resident as in the single kernel (N = 131072,
+// width 8: 74 us with all sums in four lanes).
 constexpr int GB_LANES = 4;
 template <int NV>
 __global__ void k_gsum_b(const GsumOut* __restrict__ outs, int nouts, const F2* __restrict__ pscale,
                          const float2* __restrict__ partial, F2 alpha, float2* __restrict__ v) {
+  constexpr int KL = NV / 2, LANES = GB_LANES * KL;
   pdl_trigger();
   pdl_wait();
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const int64_t i = t / GB_LANES;
-  const int k = (int)(t % GB_LANES);
+  const int64_t i = t / LANES;
+  const int k = (int)(t % LANES) / KL, kp = (int)(t % KL);
   const bool on = i < nouts;
   GsumOut O{};
   if (on) O = outs[i];
-  FF s[NV];
-#pragma unroll
-  for (int u = 0; u < NV; ++u) s[u] = FF{0.f, 0.f};
+  FF s0 = {0.f, 0.f}, s1 = {0.f, 0.f};
+  const float4* src = reinterpret_cast<const float4*>(partial) + kp;
+  if (O.flags & 2) {
 #pragma unroll 2
-  for (int p = O.p0 + k; p < O.p1; p += GB_LANES) {
-    const float4* src = reinterpret_cast<const float4*>(partial + (int64_t)p * NV);
-    float4 x[NV / 2];
-#pragma unroll
-    for (int u = 0; u < NV / 2; ++u) x[u] = __ldcg(src + u);
-    const bool ws = (O.flags & 2) != 0;
-    const F2 w = ws ? pscale[O.ps + (p - O.p0)] : F2{1.f, 0.f};
-#pragma unroll
-    for (int u = 0; u < NV; ++u) {
-      FF a = (u & 1) ? FF{x[u / 2].z, x[u / 2].w} : FF{x[u / 2].x, x[u / 2].y};
-      if (ws) a = ff_mul(a, FF{w.hi, w.lo});
-      s[u] = ff_add(s[u], a);
+    for (int p = O.p0 + k; p < O.p1; p += GB_LANES) {
+      const float4 x = __ldcg(src + (int64_t)p * KL);
+      const F2 w = pscale[O.ps + (p - O.p0)];
+      s0 = ff_add(s0, ff_mul(FF{x.x, x.y}, FF{w.hi, w.lo}));
+      s1 = ff_add(s1, ff_mul(FF{x.z, x.w}, FF{w.hi, w.lo}));
+    }
+  } else {
+#pragma unroll 4
+    for (int p = O.p0 + k; p < O.p1; p += GB_LANES) {
+      const float4 x = __ldcg(src + (int64_t)p * KL);
+      s0 = ff_add(s0, FF{x.x, x.y});
+      s1 = ff_add(s1, FF{x.z, x.w});
     }
   }
 #pragma unroll
-  for (int m = GB_LANES / 2; m >= 1; m >>= 1)   // whole warps: every lane takes part
-#pragma unroll
-    for (int u = 0; u < NV; ++u) {
-      const float hi = __shfl_xor_sync(HM_FULL, s[u].hi, m);
-      const float lo = __shfl_xor_sync(HM_FULL, s[u].lo, m);
-      s[u] = (k & m) ? ff_add(FF{hi, lo}, s[u]) : ff_add(s[u], FF{hi, lo});
-    }
-  if (!on) return;
-#pragma unroll
-  for (int u = 0; u < NV; ++u) {
-    if (u % GB_LANES != k) continue;
-    FF z = ff_mul(s[u], FF{O.scale.hi, O.scale.lo});
-    if (O.flags & 1) z = ff_mul(z, FF{alpha.hi, alpha.lo});
-    v[(int64_t)O.out * NV + u] = make_float2(z.hi, z.lo);
+  for (int m = GB_LANES / 2; m >= 1; m >>= 1) {   // whole warps: every lane takes part
+    const FF a = {__shfl_xor_sync(HM_FULL, s0.hi, m * KL), __shfl_xor_sync(HM_FULL, s0.lo, m * KL)};
+    const FF b = {__shfl_xor_sync(HM_FULL, s1.hi, m * KL), __shfl_xor_sync(HM_FULL, s1.lo, m * KL)};
+    s0 = (k & m) ? ff_add(a, s0) : ff_add(s0, a);
+    s1 = (k & m) ? ff_add(b, s1) : ff_add(s1, b);
   }
+  if (!on || k != 0) return;
+  s0 = ff_mul(s0, FF{O.scale.hi, O.scale.lo});
+  s1 = ff_mul(s1, FF{O.scale.hi, O.scale.lo});
+  if (O.flags & 1) {
+    s0 = ff_mul(s0, FF{alpha.hi, alpha.lo});
+    s1 = ff_mul(s1, FF{alpha.hi, alpha.lo});
+  }
+  reinterpret_cast<float4*>(v)[(int64_t)O.out * KL + kp] = make_float4(s0.hi, s0.lo, s1.hi, s1.lo);
 }
 
 // ---------------------------------------------------------------- column dots
@@ -303,7 +306,6 @@ __global__ void __launch_bounds__(BCfg<TIER, NV>::CW * 32, 1)
     mbar_init_fence();
   }
   __syncwarp();
-  pdl_wait();
   const uint32_t sring = smem_u32(ring);
   const ItemCopy zero{0, 0, -1, 0};
   ItemCopy dc = lane < n ? cps[p0 + lane] : zero;
@@ -311,7 +313,8 @@ __global__ void __launch_bounds__(BCfg<TIER, NV>::CW * 32, 1)
   int dbase = 0, issued = 0;
   const uint64_t pol = policy_evict_first();
   int32_t last_vin = -1, last_rows = -1;
-  auto issue = [&](int i) {   // all lanes; copies piece i (and its input segment if new)
+  // all lanes; copies piece i (and, if `withx`, its input segment when it is a new one); returns whether it is
+  auto issue = [&](int i, bool withx) {
     if (i - dbase >= 32) {
       dc = dn;
       dbase += 32;
@@ -332,11 +335,19 @@ __global__ void __launch_bounds__(BCfg<TIER, NV>::CW * 32, 1)
       fence_proxy_async();
       mbar_expect_tx(&bars[s], pb + xb);
       bulk_g2s_hint(st, pay + (uint64_t)off16 * 16u, pb, &bars[s], pol);
-      if (newx) bulk_g2s(st + STAGE_BYTES, vec + (int64_t)vin * NV, xb, &bars[s]);
+      if (newx && withx) bulk_g2s(st + STAGE_BYTES, vec + (int64_t)vin * NV, xb, &bars[s]);
     }
     issued = i + 1;
+    return newx;
   };
-  for (int i = 0; i < NS && i < n; ++i) issue(i);
+  unsigned xs = 0;
+  for (int i = 0; i < NS && i < n; ++i) xs |= (unsigned)issue(i, false) << i;
+  pdl_wait();   // the input segments come from the previous kernel
+  for (int i = 0; i < NS && i < n; ++i) {
+    const int32_t vin = __shfl_sync(HM_FULL, dc.vin, i), nrows = __shfl_sync(HM_FULL, dc.nrows, i);
+    if (lane == 0 && (xs >> i & 1u))
+      bulk_g2s(ring + i * SSTR + STAGE_BYTES, vec + (int64_t)vin * NV, (uint32_t)nrows * NV * 8u, &bars[i]);
+  }
   float2 xh[NV][4], xl[TIER == TIER_FF ? NV : 1][4];
   int32_t xv = -1, xr = -1;
   for (int i = 0; i < n; ++i) {
@@ -391,7 +402,7 @@ __global__ void __launch_bounds__(BCfg<TIER, NV>::CW * 32, 1)
     }
     }
     __syncwarp();
-    if (issued < n) issue(issued);
+    if (issued < n) issue(issued, true);
   }
 }
 
@@ -544,7 +555,7 @@ __global__ void __launch_bounds__(BCfg<TIER, NV>::RW * 32, 1)
       src[u] = j < nc ? (fan_run ? __ldg(A.fan + (moff - A.fan_base) + j) : moff + j) : 0;
     }
   };
-  auto issue = [&](int i) {   // src holds piece i's sources
+  auto payload = [&](int i) {
     if (i - dbase >= 32) {
       dc = dn;
       dbase += 32;
@@ -554,21 +565,24 @@ __global__ void __launch_bounds__(BCfg<TIER, NV>::RW * 32, 1)
     const uint32_t off16 = __shfl_sync(HM_FULL, dc.off16, sl), bf = __shfl_sync(HM_FULL, dc.bytes_flags, sl);
     const int32_t sp = __shfl_sync(HM_FULL, dc.split_part, sl);
     const int s = i % NS;
-    uint8_t* st = ring + s * SSTR;
-    const int nc = (int)(bf >> 24);
     const uint32_t pb = pad16u(bf & 0xffffu);
     fence_proxy_async();
     if (lane == 0) {
       info[s] = make_int4((int)((bf >> 16) & 0xffu), sp, 0, 0);
       mbar_expect_tx(&bars[s], pb);
-      bulk_g2s_hint(st, A.pay + (uint64_t)off16 * 16u, pb, &bars[s], pol);
+      bulk_g2s_hint(ring + s * SSTR, A.pay + (uint64_t)off16 * 16u, pb, &bars[s], pol);
     }
     __syncwarp();
+    issued = i + 1;
+  };
+  auto rows = [&](int i) {   // src holds piece i's sources
+    const int s = i % NS;
+    const int nc = (int)(__shfl_sync(HM_FULL, dc.bytes_flags, i - dbase) >> 24);
 #pragma unroll
     for (int u = 0; u < 2; ++u) {
       const int j = lane + 32 * u;
       if (j < nc) {
-        const uint32_t dst = smem_u32(st + STAGE_BYTES) + (uint32_t)(j * NV * 8);
+        const uint32_t dst = sring + (uint32_t)(s * SSTR + STAGE_BYTES + j * NV * 8);
         const float2* row = A.vec + (int64_t)src[u] * NV;
 #pragma unroll
         for (int c = 0; c < NV / 2; ++c)
@@ -577,11 +591,11 @@ __global__ void __launch_bounds__(BCfg<TIER, NV>::RW * 32, 1)
     }
     cp_arrive(&bars[s]);
     if (i + 1 < n) sources(i + 1);
-    issued = i + 1;
   };
   sources(0);
+  for (int i = 0; i < NS && i < n; ++i) payload(i);
   pdl_wait();   // multipliers and outputs depend on the previous kernels
-  for (int i = 0; i < NS && i < n; ++i) issue(i);
+  for (int i = 0; i < NS && i < n; ++i) rows(i);
   float2 ahi[NV][4], alo[NV][4];
 #pragma unroll
   for (int k = 0; k < NV; ++k)
@@ -654,7 +668,10 @@ __global__ void __launch_bounds__(BCfg<TIER, NV>::RW * 32, 1)
       }
     }
     __syncwarp();
-    if (issued < n) issue(issued);
+    if (issued < n) {
+      payload(issued);
+      rows(issued - 1);
+    }
   }
 }
 
@@ -697,7 +714,7 @@ cudaError_t launch_gather_b(int nv, const double* x, int64_t ldx, int r, const i
 cudaError_t launch_gsum_b(int nv, const GsumOut* outs, int nouts, const F2* pscale, const float2* partial, F2 alpha,
                           float2* v, cudaStream_t st) {
   if (nouts <= 0) return cudaSuccess;
-  const unsigned grid = (unsigned)(((int64_t)nouts * GB_LANES + 255) / 256);
+  const unsigned grid = (unsigned)(((int64_t)nouts * GB_LANES * (nv / 2) + 255) / 256);
   switch (nv) {
     case 2: return launch_pdl(k_gsum_b<2>, grid, 256, 0, st, outs, nouts, pscale, partial, alpha, v);
     case 4: return launch_pdl(k_gsum_b<4>, grid, 256, 0, st, outs, nouts, pscale, partial, alpha, v);

@@ -58,7 +58,7 @@ constexpr int RS_CFG_STAGES[NCFG] = {2, 3, 4};
 // launches into MR_CDOT_RANGES ranges per SM.  Chunks of at most MP_ROWS rows
 // may run on the FP32-pipe kernel; wider ones run on the tensor-core kernel.
 constexpr int RP = 32;
-constexpr int MP_PAIRS = 4;
+constexpr int MP_PAIRS = 6;
 constexpr int MP_ROWS = 64;
 constexpr int MR_CDOT_RANGES = 16;
 constexpr int MR_SHAPE = NCFG;

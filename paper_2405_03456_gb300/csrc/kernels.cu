@@ -156,7 +156,9 @@ struct CsArgs {
 // when it changes), decoded and reduced.  it counts the stages this warp has
 // used before (their mbarrier phases) and is advanced.  Returns false if a
 // copy did not arrive in time (error latched).
-template <int TIER, int NS, int SSTR>
+// PDL: the pieces of the first stages are copied before the kernel waits for its
+// predecessor (only the input segments depend on it).
+template <int TIER, int NS, int SSTR, bool PDL = false>
 __device__ __forceinline__ bool cs_range(const CsArgs& A, int p0, int n, uint8_t* ring, uint64_t* bars, int lane,
                                          uint32_t& it) {
   const uint32_t sring = smem_u32(ring);
@@ -168,7 +170,13 @@ __device__ __forceinline__ bool cs_range(const CsArgs& A, int p0, int n, uint8_t
   int dbase = 0, issued = 0;
   const uint64_t pol = policy_evict_first();
   int32_t last_vin = -1, last_rows = -1;   // input segment of the last issued piece
-  auto issue = [&](int i) {   // all lanes; copies piece i (and its input segment if new) into stage (it0 + i) % NS
+  auto copy_x = [&](uint32_t st_i, int32_t vin, int32_t nrows) {   // lane 0; the input segment of a stage's piece
+    const int64_t x0 = (int64_t)vin & ~int64_t(1);
+    bulk_g2s(ring + st_i * SSTR + A_XOFF, A.vec + x0, pad16u((uint32_t)((vin - x0) + nrows) * 8u), &bars[st_i]);
+  };
+  // all lanes; copies piece i (and, if `withx`, its input segment when it is a new one) into stage (it0 + i) % NS;
+  // returns whether it has a new input segment
+  auto issue = [&](int i, bool withx) {
     if (i - dbase >= 32) {
       dc = dn;
       dbase += 32;
@@ -192,11 +200,22 @@ __device__ __forceinline__ bool cs_range(const CsArgs& A, int p0, int n, uint8_t
       fence_proxy_async();
       mbar_expect_tx(bar, pb + xb);
       bulk_g2s_hint(st, A.pay + (uint64_t)off16 * 16u, pb, bar, pol);
-      if (newx) bulk_g2s(st + A_XOFF, A.vec + x0, xb, bar);
+      if (newx && withx) copy_x(st_i, vin, nrows);
     }
     issued = i + 1;
+    return newx;
   };
-  for (int i = 0; i < NS && i < n; ++i) issue(i);
+  if constexpr (PDL) {
+    unsigned xs = 0;
+    for (int i = 0; i < NS && i < n; ++i) xs |= (unsigned)issue(i, false) << i;
+    pdl_wait();   // the input segments come from the previous kernel
+    for (int i = 0; i < NS && i < n; ++i) {
+      const int32_t vin = __shfl_sync(HM_FULL, dc.vin, i), nrows = __shfl_sync(HM_FULL, dc.nrows, i);
+      if (lane == 0 && (xs >> i & 1u)) copy_x((it0 + (uint32_t)i) % NS, vin, nrows);
+    }
+  } else {
+    for (int i = 0; i < NS && i < n; ++i) issue(i, true);
+  }
   constexpr int RL = RPL;   // rows per lane
   float xh[RL], xl[RL];
   int32_t xv = -1, xr = -1;
@@ -237,7 +256,7 @@ __device__ __forceinline__ bool cs_range(const CsArgs& A, int p0, int n, uint8_t
         latch_error(A.err, 1);
     }
     __syncwarp();
-    if (issued < n) issue(issued);
+    if (issued < n) issue(issued, true);
   }
   it = it0 + (uint32_t)n;
   return true;
@@ -262,10 +281,9 @@ __global__ void __launch_bounds__(NW * 32, 1)
     mbar_init_fence();
   }
   __syncwarp();
-  pdl_wait();   // the input segments come from the previous kernel
   const CsArgs A{cps, pay, vec, alpha, partial, vout, err};
   uint32_t it = 0;
-  cs_range<TIER, NS, A_STAGE>(A, p0, n, ring, bars, lane, it);
+  cs_range<TIER, NS, A_STAGE, true>(A, p0, n, ring, bars, lane, it);
 }
 
 // ---------------------------------------------------------------- row chunks (phase C)
@@ -396,8 +414,10 @@ __device__ __forceinline__ bool wait_version(const DfArgs& D, int c, int v) {
 // DF (persistent launches): a piece's payload is copied at once, its
 // multipliers only after the chunks it depends on have reached their versions;
 // every emit of a coefficient chunk then publishes the next version.
+// PDL: the pieces of the first stages are copied before the kernel waits for its
+// predecessor (only the multipliers and the outputs depend on it).
 // Returns false if a copy or a dependency did not arrive in time (error latched).
-template <int TIER, int MODE, int NS, bool DF = false>
+template <int TIER, int MODE, int NS, bool DF = false, bool PDL = false>
 __device__ __forceinline__ bool rs_range(const RsArgs& A, int p0, int n, uint8_t* ring, int4* info,
                                          uint64_t* bars, int lane, uint32_t& it, const DfArgs* D = nullptr) {
   const uint32_t sring = smem_u32(ring);
@@ -407,7 +427,12 @@ __device__ __forceinline__ bool rs_range(const RsArgs& A, int p0, int n, uint8_t
   int dbase = 0, issued = 0;
   const uint64_t pol = policy_evict_first();
   const uint32_t it0 = it;
-  auto issue = [&](int i) {   // all lanes; copies piece i and its multipliers into stage (it0 + i) % NS
+  auto copy_m = [&](uint32_t st_i, int32_t moff, uint32_t nc) {   // lane 0; the multipliers of a stage's piece
+    const int64_t m0 = (int64_t)moff & ~int64_t(1);
+    if (nc) bulk_g2s(ring + st_i * C_STAGE + C_MOFF, A.vec + m0, pad16u((uint32_t)((moff - m0) + nc) * 8u), &bars[st_i]);
+  };
+  // all lanes; copies piece i and (if `withm`) its multipliers into stage (it0 + i) % NS
+  auto issue = [&](int i, bool withm) {
     if (i - dbase >= 32) {
       dc = dn;
       dbase += 32;
@@ -437,12 +462,22 @@ __device__ __forceinline__ bool rs_range(const RsArgs& A, int p0, int n, uint8_t
         asm volatile("fence.proxy.async.global;" ::: "memory");   // the multipliers were written by other SMs
       }
       info[st_i] = make_int4((int)((bf >> 16) & 0xffu), sp, moff & 1, ce);
-      if (mb) bulk_g2s(st + C_MOFF, A.vec + m0, mb, bar);   // issued even after a failed wait: the stage completes
+      if (withm) copy_m(st_i, moff, nc);   // issued even after a failed wait: the stage completes
     }
     if constexpr (DF) __syncwarp();   // lane 0's acquires before the lanes' reads of this piece's chunk
     issued = i + 1;
   };
-  for (int i = 0; i < NS && i < n; ++i) issue(i);
+  if constexpr (PDL) {
+    for (int i = 0; i < NS && i < n; ++i) issue(i, false);
+    pdl_wait();
+    for (int i = 0; i < NS && i < n; ++i) {
+      const int32_t moff = __shfl_sync(HM_FULL, dc.moff, i);
+      const uint32_t bf = __shfl_sync(HM_FULL, dc.bytes_flags, i);
+      if (lane == 0) copy_m((it0 + (uint32_t)i) % NS, moff, bf >> 24);
+    }
+  } else {
+    for (int i = 0; i < NS && i < n; ++i) issue(i, true);
+  }
   constexpr int RL = RPL;   // rows per lane
   float2 ahi[4], alo[4];     // float-float row sums, rows (2k, 2k+1)
 #pragma unroll
@@ -511,7 +546,7 @@ __device__ __forceinline__ bool rs_range(const RsArgs& A, int p0, int n, uint8_t
       }
     }
     __syncwarp();
-    if (issued < n) issue(issued);
+    if (issued < n) issue(issued, true);
   }
   it = it0 + (uint32_t)n;
   return true;
@@ -543,9 +578,8 @@ __global__ void __launch_bounds__(NW * 32, 1)
   int4* info;
   uint64_t* bars;
   rs_ring_init<NW, NS>(ring, info, bars, warp, lane);
-  pdl_wait();   // multipliers and outputs depend on the previous kernels
   uint32_t it = 0;
-  rs_range<TIER, MODE, NS>(A, p0, n, ring, info, bars, lane, it);
+  rs_range<TIER, MODE, NS, false, true>(A, p0, n, ring, info, bars, lane, it);
 }
 
 // ---------------------------------------------------------------- persistent phases

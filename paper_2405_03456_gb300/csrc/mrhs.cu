@@ -13,59 +13,72 @@
 #include <cstdint>
 #include <cuda_runtime.h>
 
-#include "decode.cuh"
+#include "stream.cuh"
 
 namespace hm {
 
 __device__ __forceinline__ uint32_t pad16m(uint32_t x) { return (x + 15u) & ~15u; }
 
 // ---------------------------------------------------------------- gather, segment sums
+// Four right-hand sides per thread (independent loads, one 16-byte store): one per
+// thread left the kernels with too few loads in flight (N = 131072, 32 columns:
+// gather 28 us, segment sums 107 us).
 // v[i * RP + k] = x[perm[i] + k * ldx] (FP32 hi part), k < r; zero for k >= r.
+constexpr int KQ = RP / 4;
 __global__ void k_gather_mr(const double* __restrict__ x, int64_t ldx, int r, const int32_t* __restrict__ perm, int n,
                             float* __restrict__ v) {
+  pdl_trigger();
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= (int64_t)n * RP) return;
-  const int i = (int)(t / RP), k = (int)(t % RP);
-  v[t] = k < r ? (float)x[(int64_t)perm[i] + k * ldx] : 0.0f;
+  const int i = (int)(t / KQ), k = 4 * (int)(t % KQ);
+  const double* xi = x + (i < n ? __ldg(perm + i) : 0);
+  pdl_wait();   // x may be the previous kernel's result, and that kernel may still read v
+  if (i >= n) return;
+  float f[4];
+#pragma unroll
+  for (int u = 0; u < 4; ++u) f[u] = k + u < r ? (float)xi[(int64_t)(k + u) * ldx] : 0.0f;
+  *reinterpret_cast<float4*>(v + 4 * t) = make_float4(f[0], f[1], f[2], f[3]);
 }
 
 __global__ void k_gsum_mr(const GsumOut* __restrict__ outs, int nouts, const F2* __restrict__ pscale,
                           const float* __restrict__ partial, F2 alpha, float* __restrict__ v) {
+  pdl_trigger();
+  pdl_wait();
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= (int64_t)nouts * RP) return;
-  const GsumOut O = outs[t / RP];
-  const int k = (int)(t % RP);
+  if (t >= (int64_t)nouts * KQ) return;
+  const GsumOut O = outs[t / KQ];
+  const int kq = (int)(t % KQ);
   const bool ws = (O.flags & 2) != 0;
-  FF s = {0.f, 0.f};
-  // partials in order p0, p0 + 1, ...; four loads in flight per step
-  int p = O.p0;
-  for (; p + 4 <= O.p1; p += 4) {
-    float x[4];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) x[u] = __ldcs(partial + (int64_t)(p + u) * RP + k);
-    if (ws) {
-      F2 wv[4];
-#pragma unroll
-      for (int u = 0; u < 4; ++u) wv[u] = pscale[O.ps + (p + u - O.p0)];
-#pragma unroll
-      for (int u = 0; u < 4; ++u) s = ff_add(s, ff_mul(FF{x[u], 0.f}, FF{wv[u].hi, wv[u].lo}));
-    } else {
-#pragma unroll
-      for (int u = 0; u < 4; ++u) s = ff_add_f(s, x[u]);
-    }
-  }
-  for (; p < O.p1; ++p) {
-    const float x = __ldcs(partial + (int64_t)p * RP + k);
-    if (ws) {
+  const float4* src = reinterpret_cast<const float4*>(partial) + kq;
+  FF s[4] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
+  // partials in order p0, p0 + 1, ... (unrolled: several loads in flight)
+  if (ws) {
+#pragma unroll 2
+    for (int p = O.p0; p < O.p1; ++p) {
+      const float4 x = __ldcs(src + (int64_t)p * KQ);
       const F2 w = pscale[O.ps + (p - O.p0)];
-      s = ff_add(s, ff_mul(FF{x, 0.f}, FF{w.hi, w.lo}));
-    } else {
-      s = ff_add_f(s, x);
+      s[0] = ff_add(s[0], ff_mul(FF{x.x, 0.f}, FF{w.hi, w.lo}));
+      s[1] = ff_add(s[1], ff_mul(FF{x.y, 0.f}, FF{w.hi, w.lo}));
+      s[2] = ff_add(s[2], ff_mul(FF{x.z, 0.f}, FF{w.hi, w.lo}));
+      s[3] = ff_add(s[3], ff_mul(FF{x.w, 0.f}, FF{w.hi, w.lo}));
+    }
+  } else {
+#pragma unroll 4
+    for (int p = O.p0; p < O.p1; ++p) {
+      const float4 x = __ldcs(src + (int64_t)p * KQ);
+      s[0] = ff_add_f(s[0], x.x);
+      s[1] = ff_add_f(s[1], x.y);
+      s[2] = ff_add_f(s[2], x.z);
+      s[3] = ff_add_f(s[3], x.w);
     }
   }
-  s = ff_mul(s, FF{O.scale.hi, O.scale.lo});
-  if (O.flags & 1) s = ff_mul(s, FF{alpha.hi, alpha.lo});
-  v[(int64_t)O.out * RP + k] = s.hi + s.lo;
+  float o[4];
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    FF z = ff_mul(s[u], FF{O.scale.hi, O.scale.lo});
+    if (O.flags & 1) z = ff_mul(z, FF{alpha.hi, alpha.lo});
+    o[u] = z.hi + z.lo;
+  }
+  *reinterpret_cast<float4*>(v + ((int64_t)O.out * KQ + kq) * 4) = make_float4(o[0], o[1], o[2], o[3]);
 }
 
 // ---------------------------------------------------------------- row chunks
@@ -74,13 +87,21 @@ __global__ void k_gsum_mr(const GsumOut* __restrict__ outs, int nouts, const F2*
 // each multiplier row -- the RP values of the coefficient it stands for -- by
 // 16-byte cp.async); warp wi of the pair takes rows 32 wi .. 32 wi + 31 of every
 // piece and all RP right-hand sides.  Lane (g = lane / 4, tq = lane % 4) holds
-// rows 32 wi + 4 g .. + 3 and right-hand sides 8 nt + 2 tq + {0, 1}, nt < NT.
+// rows 32 wi + 4 g .. + 3 and right-hand sides 8 tq + 2 nt + {0, 1}, nt < NT.
+// What bounds it: instructions, not bytes (a value is 32 multiply-adds, 16 paired
+// ones of a lane's 4 rows x 8 right-hand sides a column).  Decoding in every lane
+// that multiplies took more of them than the products; here the four lanes tq of
+// a row group decode one column each of the next four and share the values
+// through shared memory.  Six pairs per SM with two stages each (four with three
+// before: 8 warps an SM could not hide the latency of their own chains).
 constexpr int NT = RP / 8;
-constexpr int MP_NS = 3;                                   // stages per pair
+constexpr int MP_NS = 2;                                   // stages per pair
 constexpr int MP_TP = RP * 4 + 16;                         // multiplier row pitch in a stage (bytes)
 constexpr int MP_STAGE = STAGE_BYTES + PIECE_MAX_COLS * MP_TP;
 constexpr int MP_THREADS = MP_PAIRS * 64;
-constexpr size_t MP_SMEM = (size_t)MP_PAIRS * MP_NS * MP_STAGE + (size_t)MP_PAIRS * MP_NS * 8;
+constexpr int MP_SCC = 32 * 4 + 32;                        // pitch of a decoded column (16-byte stores of 4 lanes tq: distinct banks)
+constexpr int MP_SCR = 2 * 4 * MP_SCC;                     // decoded values of a warp: 2 turns x 4 columns x 32 rows
+constexpr size_t MP_SMEM = (size_t)MP_PAIRS * MP_NS * MP_STAGE + (size_t)MP_PAIRS * 2 * MP_SCR + (size_t)MP_PAIRS * MP_NS * 8;
 static_assert(MP_STAGE % 128 == 0, "stage alignment");
 static_assert(MP_SMEM <= 227 * 1024, "row-chunk pairs per block");
 
@@ -99,10 +120,11 @@ __device__ __forceinline__ bool pair_any(int bid, bool v) {
 // One piece for warp wi of the pair on the FP32 pipes: every product is one
 // FP32 FMA (FFMA2 over right-hand-side pairs), as in the single-RHS kernels,
 // summed per piece in FP32 and folded into the float-float sums fhi / flo
-// [mt][nt][h] of rows 32 wi + 4 g + 2 mt + h, right-hand sides 8 nt + 2 tq +
-// {0, 1}.  Per column the lane decodes its 4 codes and reads its 8 multipliers.
+// [mt][nt][h] of rows 32 wi + 4 g + 2 mt + h, right-hand sides 8 tq + 2 nt +
+// {0, 1}.  Turns of four columns: lane (g, tq) decodes its row group's 4 codes of
+// column j + tq into the warp's scratch scr, then multiplies all four.
 template <int F, int B>
-__device__ __forceinline__ void ms_piece(uint32_t sa, const PieceHdr& H, F2 alpha_ff, int wi, int lane,
+__device__ __forceinline__ void ms_piece(uint32_t sa, uint32_t scr, const PieceHdr& H, F2 alpha_ff, int wi, int lane,
                                          float2 (&fhi)[2][NT][2], float2 (&flo)[2][NT][2]) {
   const int R = H.nrows, nc = H.ncols;
   const bool tile = (H.flags & PH_TILE) != 0;
@@ -110,41 +132,60 @@ __device__ __forceinline__ void ms_piece(uint32_t sa, const PieceHdr& H, F2 alph
   const uint32_t cm = sa + (uint32_t)sizeof(PieceHdr);
   const int g = lane >> 2, tq = lane & 3;
   const uint32_t cb = cm + (tile ? 0u : pad8u(2u * nc)) + (uint32_t)((32 * wi + 4 * g) * B);
-  const uint32_t tv = sa + STAGE_BYTES + 8u * tq;
+  const uint32_t tv = sa + STAGE_BYTES + 32u * tq;
+  const uint32_t sw = scr + (uint32_t)(tq * MP_SCC + g * 16), sr = scr + (uint32_t)(g * 16);
   const int e_t = H.em & 0xff, m_t = H.em >> 8;
   float2 acc[4][NT];
 #pragma unroll
   for (int u = 0; u < 4; ++u)
 #pragma unroll
     for (int nt = 0; nt < NT; ++nt) acc[u][nt] = make_float2(0.f, 0.f);
-#pragma unroll 2
-  for (int j = 0; j < nc; ++j) {
-    int e = e_t, m = m_t;
-    if constexpr (F == 2) {
-      if (!tile) {
-        const uint32_t em = lds32((cm + 2u * j) & ~3u) >> (16u * (j & 1));
-        e = em & 0xff;
-        m = (em >> 8) & 0xff;
+  uint32_t buf = 0;
+#pragma unroll 1
+  for (int j0 = 0; j0 < nc; j0 += 4, buf = 4u * MP_SCC - buf) {
+    const int jd = j0 + tq;
+    if (jd < nc) {
+      int e = e_t, m = m_t;
+      if constexpr (F == 2) {
+        if (!tile) {
+          const uint32_t em = lds32((cm + 2u * jd) & ~3u) >> (16u * (jd & 1));
+          e = em & 0xff;
+          m = (em >> 8) & 0xff;
+        }
       }
+      uint32_t w[B];
+#pragma unroll
+      for (int b = 0; b < B; ++b) w[b] = lds32(cb + (uint32_t)jd * stride + 4u * b);
+      float v[4], l[4];
+      decode4<TIER_F32, F, B>(w, e, m, v, l);
+      asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(sw + buf), "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3])
+                   : "memory");
     }
-    uint32_t w[B];
+    __syncwarp();   // (this buffer is written again two turns later, behind the next turn's barrier)
+    auto column = [&](int c) {
+      const uint4 vq = lds128(sr + buf + (uint32_t)(MP_SCC * c));
+      const float v[4] = {__uint_as_float(vq.x), __uint_as_float(vq.y), __uint_as_float(vq.z), __uint_as_float(vq.w)};
+      const uint4 q0 = lds128(tv + (uint32_t)(j0 + c) * MP_TP), q1 = lds128(tv + (uint32_t)(j0 + c) * MP_TP + 16u);
+      const float2 t[NT] = {make_float2(__uint_as_float(q0.x), __uint_as_float(q0.y)),
+                            make_float2(__uint_as_float(q0.z), __uint_as_float(q0.w)),
+                            make_float2(__uint_as_float(q1.x), __uint_as_float(q1.y)),
+                            make_float2(__uint_as_float(q1.z), __uint_as_float(q1.w))};
 #pragma unroll
-    for (int b = 0; b < B; ++b) w[b] = lds32(cb + (uint32_t)j * stride + 4u * b);
-    float v[4], l[4];
-    decode4<TIER_F32, F, B>(w, e, m, v, l);
-    float2 t[NT];
+      for (int u = 0; u < 4; ++u) {
+        const float2 vv = make_float2(v[u], v[u]);
 #pragma unroll
-    for (int nt = 0; nt < NT; ++nt) {
-      const uint2 q = lds64(tv + (uint32_t)j * MP_TP + 32u * nt);
-      t[nt] = make_float2(__uint_as_float(q.x), __uint_as_float(q.y));
-    }
+        for (int nt = 0; nt < NT; ++nt) acc[u][nt] = __ffma2_rn(vv, t[nt], acc[u][nt]);
+      }
+    };
+    if (j0 + 4 <= nc) {   // four columns: their loads in flight together
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const float2 vv = make_float2(v[u], v[u]);
-#pragma unroll
-      for (int nt = 0; nt < NT; ++nt) acc[u][nt] = __ffma2_rn(vv, t[nt], acc[u][nt]);
+      for (int c = 0; c < 4; ++c) column(c);
+    } else {
+#pragma unroll 1
+      for (int c = 0; c < nc - j0; ++c) column(c);
     }
   }
+  __syncwarp();   // the scratch is free for the next piece
   float2 sc2 = make_float2(1.f, 1.f);
   if (tile) {
     FF f = {H.scale.hi, H.scale.lo};
@@ -171,13 +212,16 @@ __global__ void __launch_bounds__(MP_THREADS, 1)
   extern __shared__ __align__(128) uint8_t smem[];
   __shared__ int4 info[MP_PAIRS][MP_NS];
   __shared__ int s_last[MP_PAIRS];
+  pdl_trigger();
   const int pair = threadIdx.x >> 6, wi = (threadIdx.x >> 5) & 1, lane = threadIdx.x & 31;
   const int gp = blockIdx.x * MP_PAIRS + pair;
   if (gp >= nrange) return;   // the whole pair
   const int p0 = wbeg[gp], n = wbeg[gp + 1] - p0;
   if (n <= 0) return;
   uint8_t* ring = smem + (size_t)pair * MP_NS * MP_STAGE;
-  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + (size_t)MP_PAIRS * MP_NS * MP_STAGE) + pair * MP_NS;
+  uint8_t* scratch = smem + (size_t)MP_PAIRS * MP_NS * MP_STAGE;
+  const uint32_t scr = smem_u32(scratch) + (uint32_t)((2 * pair + wi) * MP_SCR);
+  uint64_t* bars = reinterpret_cast<uint64_t*>(scratch + (size_t)MP_PAIRS * 2 * MP_SCR) + pair * MP_NS;
   const int bid = 1 + pair;
   const uint64_t pol = policy_evict_first();
   // warp 0 of the pair issues the copies; its lanes hold the copy descriptors 32 at a time
@@ -239,8 +283,10 @@ __global__ void __launch_bounds__(MP_THREADS, 1)
     }
     __syncwarp();
     sources(0);
-    for (int i = 0; i < MP_NS && i < n; ++i) issue(i);
   }
+  pdl_wait();   // multipliers and outputs depend on the previous kernels
+  if (wi == 0)
+    for (int i = 0; i < MP_NS && i < n; ++i) issue(i);
   pair_sync(bid);   // the barriers are initialised before warp 1 waits on them
   const int g = lane >> 2, tq = lane & 3;
   float2 fhi[2][NT][2], flo[2][NT][2];
@@ -294,7 +340,7 @@ __global__ void __launch_bounds__(MP_THREADS, 1)
     if (32 * wi < R) {
       switch (H.fb) {
 #define HM_MP(FF_, BB_) \
-  case ((FF_) << 4) | (BB_): ms_piece<FF_, BB_>(sa, H, alpha_ff, wi, lane, fhi, flo); break;
+  case ((FF_) << 4) | (BB_): ms_piece<FF_, BB_>(sa, scr, H, alpha_ff, wi, lane, fhi, flo); break;
         HM_FORMATS(HM_MP)
 #undef HM_MP
         default:
@@ -316,7 +362,7 @@ __global__ void __launch_bounds__(MP_THREADS, 1)
             if (row < R) {
 #pragma unroll
               for (int nt = 0; nt < NT; ++nt) {
-                const int k = 8 * nt + 2 * tq;
+                const int k = 8 * tq + 2 * nt;
                 *reinterpret_cast<float4*>(mine + row * RP + k) =
                     make_float4(fhi[mt][nt][h].x, flo[mt][nt][h].x, fhi[mt][nt][h].y, flo[mt][nt][h].y);
               }
@@ -348,7 +394,7 @@ __global__ void __launch_bounds__(MP_THREADS, 1)
                 if (row < R) {
 #pragma unroll
                   for (int nt = 0; nt < NT; ++nt) {
-                    const float4 v = __ldcg(reinterpret_cast<const float4*>(src + row * RP + 8 * nt + 2 * tq));
+                    const float4 v = __ldcg(reinterpret_cast<const float4*>(src + row * RP + 8 * tq + 2 * nt));
                     const FF a = ff_add(FF{fhi[mt][nt][h].x, flo[mt][nt][h].x}, FF{v.x, v.y});
                     const FF b = ff_add(FF{fhi[mt][nt][h].y, flo[mt][nt][h].y}, FF{v.z, v.w});
                     fhi[mt][nt][h] = make_float2(a.hi, b.hi);
@@ -371,14 +417,14 @@ __global__ void __launch_bounds__(MP_THREADS, 1)
               for (int nt = 0; nt < NT; ++nt)
 #pragma unroll
                 for (int c = 0; c < 2; ++c) {
-                  const int k = 8 * nt + 2 * tq + c;
+                  const int k = 8 * tq + 2 * nt + c;
                   yo[nt][c] = (beta != 0.0 && k < r) ? y[o + (int64_t)k * ldy] : 0.0;
                 }
 #pragma unroll
               for (int nt = 0; nt < NT; ++nt)
 #pragma unroll
                 for (int c = 0; c < 2; ++c) {
-                  const int k = 8 * nt + 2 * tq + c;
+                  const int k = 8 * tq + 2 * nt + c;
                   if (k < r) {
                     const double val = ff_to_d(FF{c ? fhi[mt][nt][h].y : fhi[mt][nt][h].x,
                                                   c ? flo[mt][nt][h].y : flo[mt][nt][h].x});
@@ -390,8 +436,8 @@ __global__ void __launch_bounds__(MP_THREADS, 1)
               const F2 rsc = rowscale ? rowscale[gg] : F2{1.f, 0.f};
 #pragma unroll
               for (int nt = 0; nt < NT; ++nt) {
-                const int k0 = 8 * nt + 2 * tq;
-                const float2 old = (MODE == MODE_VEC_ADD) ? *reinterpret_cast<const float2*>(vout + (int64_t)gg * RP + k0)
+                const int k0 = 8 * tq + 2 * nt;
+                const float2 old = (MODE == MODE_VEC_ADD) ? __ldcg(reinterpret_cast<const float2*>(vout + (int64_t)gg * RP + k0))
                                                           : make_float2(0.f, 0.f);
 #pragma unroll
                 for (int c = 0; c < 2; ++c)
@@ -418,13 +464,15 @@ __global__ void __launch_bounds__(MP_THREADS, 1)
 // warp per range of pieces (its own ring of CW_NS stages, pieces only).  Lane
 // (tq = lane / 8, g = lane % 8) holds the input rows 8 g .. 8 g + 7 of the
 // segment for the right-hand sides 8 tq .. 8 tq + 7 in registers (read from
-// the panel when the segment changes); per column it decodes its 8 codes,
-// forms the 8 partial dots over its rows (FFMA2) and a reduce-scatter over the
+// the panel when the segment changes).  Turns of four columns: the lane decodes
+// its 8 rows of column j + tq into the warp's scratch, then for each of the four
+// forms the 8 partial dots over its rows (FFMA2), and a reduce-scatter over the
 // 8 lanes g leaves lane g with the column's total for right-hand side 8 tq + g
 // (each column sums its <= 64 rows in FP32, as the single-RHS kernel).
 constexpr int CW_WARPS = 16;
 constexpr int CW_NS = 2;
-constexpr size_t CW_SMEM = (size_t)CW_WARPS * CW_NS * STAGE_BYTES + (size_t)CW_WARPS * CW_NS * 8;
+constexpr int CW_SCR = 4 * 64 * 4;   // decoded values of a warp: 4 columns x 64 rows
+constexpr size_t CW_SMEM = (size_t)CW_WARPS * (CW_NS * STAGE_BYTES + CW_SCR) + (size_t)CW_WARPS * CW_NS * 8;
 static_assert(CW_SMEM <= 227 * 1024, "column-dot warps per block");
 
 // Reduce-scatter of 8 values over the 8 lanes q = lane bits 0..2 (fixed
@@ -448,7 +496,7 @@ __device__ __forceinline__ float rs8(float (&p)[8], int q) {
 }
 
 template <int F, int B>
-__device__ __forceinline__ void cw_piece(uint32_t sa, int R, int nc, int flags, const float2 (&xr)[8][4], int lane,
+__device__ __forceinline__ void cw_piece(uint32_t sa, uint32_t scr, int R, int nc, int flags, const float2 (&xr)[8][4], int lane,
                                          F2 alpha, float* __restrict__ partial, float* __restrict__ vout) {
   const int tq = lane >> 3, g = lane & 7;
   const bool fin = (flags & ITEM_FINAL) != 0;
@@ -459,37 +507,64 @@ __device__ __forceinline__ void cw_piece(uint32_t sa, int R, int nc, int flags, 
   const uint32_t cb = cm + (fin ? 16u : 8u) * nc + (uint32_t)(8 * g * B);
   const bool rows_on = 8 * g < Rp;
   const FF fa = {alpha.hi, alpha.lo};
-#pragma unroll 2
-  for (int j = 0; j < nc; ++j) {
-    int e = 0, m = 0;
-    if constexpr (F == 2) {
-      const uint32_t em = lds32(cm + 8u * j) & 0xffffu;
-      e = em & 0xff;
-      m = em >> 8;
+  // scratch: column c, rows 8 g + 4 h .. + 3 at c * 256 + h * 128 + g * 16
+  const uint32_t sw = scr + (uint32_t)(tq * 256 + g * 16), sr = scr + (uint32_t)(g * 16);
+#pragma unroll 1
+  for (int j0 = 0; j0 < nc; j0 += 4) {
+    const int jd = j0 + tq;
+    if (jd < nc) {
+      int e = 0, m = 0;
+      if constexpr (F == 2) {
+        const uint32_t em = lds32(cm + 8u * jd) & 0xffffu;
+        e = em & 0xff;
+        m = em >> 8;
+      }
+      float2 d2[4] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+      if (rows_on) decode8p<F, B>(cb + (uint32_t)jd * stride, e, m, d2);
+      asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(sw), "f"(d2[0].x), "f"(d2[0].y), "f"(d2[1].x),
+                   "f"(d2[1].y)
+                   : "memory");
+      asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(sw + 128u), "f"(d2[2].x), "f"(d2[2].y),
+                   "f"(d2[3].x), "f"(d2[3].y)
+                   : "memory");
     }
-    float2 h2[4] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-    if (rows_on) decode8p<F, B>(cb + (uint32_t)j * stride, e, m, h2);
-    float2 p2[4] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+    __syncwarp();
+    auto column = [&](int c) {
+      const int j = j0 + c;
+      const uint4 va = lds128(sr + 256u * c), vb = lds128(sr + 256u * c + 128u);
+      const float v[8] = {__uint_as_float(va.x), __uint_as_float(va.y), __uint_as_float(va.z), __uint_as_float(va.w),
+                          __uint_as_float(vb.x), __uint_as_float(vb.y), __uint_as_float(vb.z), __uint_as_float(vb.w)};
+      float2 p2[4] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
 #pragma unroll
-    for (int u = 0; u < 8; ++u) {
-      const float v = (u & 1) ? h2[u >> 1].y : h2[u >> 1].x;
-      const float2 vv = make_float2(v, v);
+      for (int u = 0; u < 8; ++u) {
+        const float2 vv = make_float2(v[u], v[u]);
 #pragma unroll
-      for (int k = 0; k < 4; ++k) p2[k] = __ffma2_rn(vv, xr[u][k], p2[k]);
-    }
-    float p[8] = {p2[0].x, p2[0].y, p2[1].x, p2[1].y, p2[2].x, p2[2].y, p2[3].x, p2[3].y};
-    const float tot = rs8(p, g);
-    const int32_t out = (int32_t)lds32(cm + 8u * j + 4u);
-    const int64_t o = (int64_t)out * RP + 8 * tq + g;
-    if (fin) {
-      const uint2 f = lds64(scl + 8u * j);
-      FF sc = {__uint_as_float(f.x), __uint_as_float(f.y)};
-      if (flags & ITEM_ALPHA) sc = ff_mul(sc, fa);
-      const FF v = ff_mul(FF{tot, 0.f}, sc);
-      vout[o] = v.hi + v.lo;
+        for (int k = 0; k < 4; ++k) p2[k] = __ffma2_rn(vv, xr[u][k], p2[k]);
+      }
+      float p[8] = {p2[0].x, p2[0].y, p2[1].x, p2[1].y, p2[2].x, p2[2].y, p2[3].x, p2[3].y};
+      const float tot = rs8(p, g);
+      const int32_t out = (int32_t)lds32(cm + 8u * j + 4u);
+      const int64_t o = (int64_t)out * RP + 8 * tq + g;
+      if (fin) {
+        const uint2 f = lds64(scl + 8u * j);
+        FF sc = {__uint_as_float(f.x), __uint_as_float(f.y)};
+        if (flags & ITEM_ALPHA) sc = ff_mul(sc, fa);
+        const FF w = ff_mul(FF{tot, 0.f}, sc);
+        vout[o] = w.hi + w.lo;
+      } else {
+        partial[o] = tot;
+      }
+    };
+    if (j0 + 4 <= nc) {   // in pairs: independent reductions
+      column(0);
+      column(1);
+      column(2);
+      column(3);
     } else {
-      partial[o] = tot;
+#pragma unroll 1
+      for (int c = 0; c < nc - j0; ++c) column(c);
     }
+    __syncwarp();   // the scratch is free for the next turn
   }
 }
 
@@ -498,13 +573,15 @@ __global__ void __launch_bounds__(CW_WARPS * 32, 1)
               const uint8_t* __restrict__ pay, const float* __restrict__ vec, F2 alpha, float* __restrict__ partial,
               float* __restrict__ vout, int* err) {
   extern __shared__ __align__(128) uint8_t smem[];
+  pdl_trigger();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int gw = blockIdx.x * CW_WARPS + warp;
   if (gw >= nrange) return;
   const int p0 = wbeg[gw], n = wbeg[gw + 1] - p0;
   if (n <= 0) return;
   uint8_t* ring = smem + (size_t)warp * CW_NS * STAGE_BYTES;
-  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + (size_t)CW_WARPS * CW_NS * STAGE_BYTES) + warp * CW_NS;
+  const uint32_t scr = smem_u32(smem + (size_t)CW_WARPS * CW_NS * STAGE_BYTES) + (uint32_t)(warp * CW_SCR);
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + (size_t)CW_WARPS * (CW_NS * STAGE_BYTES + CW_SCR)) + warp * CW_NS;
   const uint64_t pol = policy_evict_first();
   const ItemCopy zero{0, 0, -1, 0};
   ItemCopy dc = lane < n ? cps[p0 + lane] : zero;
@@ -531,7 +608,8 @@ __global__ void __launch_bounds__(CW_WARPS * 32, 1)
     mbar_init_fence();
   }
   __syncwarp();
-  for (int i = 0; i < CW_NS && i < n; ++i) issue(i);
+  for (int i = 0; i < CW_NS && i < n; ++i) issue(i);   // (packed pieces only)
+  pdl_wait();   // the input rows come from the previous kernel
   const int tq = lane >> 3, g = lane & 7;
   float2 xr[8][4];
   int32_t xv = -1, xn = -1;
@@ -557,8 +635,8 @@ __global__ void __launch_bounds__(CW_WARPS * 32, 1)
         float4 a = make_float4(0.f, 0.f, 0.f, 0.f), b = a;
         if (row < R) {
           const float4* src = reinterpret_cast<const float4*>(vec + (int64_t)(hvin + row) * RP + 8 * tq);
-          a = __ldg(src);
-          b = __ldg(src + 1);
+          a = __ldcg(src);
+          b = __ldcg(src + 1);
         }
         xr[u][0] = make_float2(a.x, a.y);
         xr[u][1] = make_float2(a.z, a.w);
@@ -570,7 +648,7 @@ __global__ void __launch_bounds__(CW_WARPS * 32, 1)
     }
     switch (fb) {
 #define HM_CW(FF_, BB_) \
-  case ((FF_) << 4) | (BB_): cw_piece<FF_, BB_>(sa, R, nc, (int)flags, xr, lane, alpha, partial, vout); break;
+  case ((FF_) << 4) | (BB_): cw_piece<FF_, BB_>(sa, scr, R, nc, (int)flags, xr, lane, alpha, partial, vout); break;
       HM_FORMATS(HM_CW)
 #undef HM_CW
       default:
@@ -596,26 +674,22 @@ cudaError_t mr_init() {
 cudaError_t launch_gather_mr(const double* x, int64_t ldx, int r, const int32_t* perm, int n, float* v,
                              cudaStream_t st) {
   if (n <= 0) return cudaSuccess;
-  const int64_t tot = (int64_t)n * RP;
-  k_gather_mr<<<(unsigned)((tot + 255) / 256), 256, 0, st>>>(x, ldx, r, perm, n, v);
-  return cudaGetLastError();
+  return launch_pdl(k_gather_mr, (unsigned)(((int64_t)n * KQ + 255) / 256), 256, 0, st, x, ldx, r, perm, n, v);
 }
 
 cudaError_t launch_gsum_mr(const GsumOut* outs, int nouts, const F2* pscale, const float* partial, F2 alpha, float* v,
                            cudaStream_t st) {
   if (nouts <= 0) return cudaSuccess;
-  const int64_t tot = (int64_t)nouts * RP;
-  k_gsum_mr<<<(unsigned)((tot + 255) / 256), 256, 0, st>>>(outs, nouts, pscale, partial, alpha, v);
-  return cudaGetLastError();
+  return launch_pdl(k_gsum_mr, (unsigned)(((int64_t)nouts * KQ + 255) / 256), 256, 0, st, outs, nouts, pscale, partial,
+                    alpha, v);
 }
 
 // nblk ranges, one per warp
 cudaError_t launch_cdot_ws(const ItemCopy* items, const int32_t* wbeg, int nblk, const uint8_t* pay, const float* vec,
                            F2 alpha, float* partial, float* vout, int* err, cudaStream_t st) {
   if (nblk <= 0) return cudaSuccess;
-  k_cdot_ws<<<(unsigned)((nblk + CW_WARPS - 1) / CW_WARPS), CW_WARPS * 32, CW_SMEM, st>>>(items, wbeg, nblk, pay, vec,
-                                                                                           alpha, partial, vout, err);
-  return cudaGetLastError();
+  return launch_pdl(k_cdot_ws, (unsigned)((nblk + CW_WARPS - 1) / CW_WARPS), CW_WARPS * 32, CW_SMEM, st, items, wbeg,
+                    nblk, pay, vec, alpha, partial, vout, err);
 }
 
 // nblk ranges, one per warp pair; chunks of at most MP_ROWS rows
@@ -625,17 +699,13 @@ cudaError_t launch_rgemv_ms(int mode, const PieceCopy* pieces, const int32_t* wb
                             const Split* splits, const int32_t* fan, int32_t fan_base, int* err, cudaStream_t st) {
   if (nblk <= 0) return cudaSuccess;
   const unsigned grid = (unsigned)((nblk + MP_PAIRS - 1) / MP_PAIRS);
-#define HM_MSG(M)                                                                                            \
-  k_rgemv_ms<M><<<grid, MP_THREADS, MP_SMEM, st>>>(pieces, wbeg, nblk, pay, vec, alpha, alpha_ff, beta, y, ldy, r, \
-                                                   perm, vout, rowscale, fix, fixcnt, splits, fan, fan_base, err)
-  if (mode == MODE_Y)
-    HM_MSG(MODE_Y);
-  else if (mode == MODE_VEC)
-    HM_MSG(MODE_VEC);
-  else
-    HM_MSG(MODE_VEC_ADD);
+#define HM_MSG(M)                                                                                             \
+  launch_pdl(k_rgemv_ms<M>, grid, MP_THREADS, MP_SMEM, st, pieces, wbeg, nblk, pay, vec, alpha, alpha_ff, beta, y, ldy, \
+             r, perm, vout, rowscale, fix, fixcnt, splits, fan, fan_base, err)
+  if (mode == MODE_Y) return HM_MSG(MODE_Y);
+  if (mode == MODE_VEC) return HM_MSG(MODE_VEC);
+  return HM_MSG(MODE_VEC_ADD);
 #undef HM_MSG
-  return cudaGetLastError();
 }
 
 }  // namespace hm

@@ -295,7 +295,7 @@ __global__ void __launch_bounds__(BCfg<TIER, NV>::CW * 32, 1)
   extern __shared__ __align__(128) uint8_t smem[];
   pdl_trigger();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int gw = blockIdx.x * NW + warp;
+  const int gw = range_of<NW>(warp, nwt);
   if (gw >= nwt) return;
   const int p0 = wbeg[gw], n = wbeg[gw + 1] - p0;
   if (n <= 0) return;
@@ -523,7 +523,7 @@ __global__ void __launch_bounds__(BCfg<TIER, NV>::RW * 32, 1)
   extern __shared__ __align__(128) uint8_t smem[];
   pdl_trigger();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int gw = blockIdx.x * NW + warp;
+  const int gw = range_of<NW>(warp, nwt);
   if (gw >= nwt) return;
   const int p0 = wbeg[gw], n = wbeg[gw + 1] - p0;
   if (n <= 0) return;
@@ -728,7 +728,7 @@ cudaError_t launch_cdot_b(int tier, int nv, const ItemCopy* items, const int32_t
   if (nw <= 0) return cudaSuccess;
 #define HM_BC(T, V)                                                                                              \
   if (tier == T && nv == V)                                                                                      \
-    return launch_pdl(k_cbatch<T, V>, (unsigned)((nw + BCfg<T, V>::CW - 1) / BCfg<T, V>::CW), BCfg<T, V>::CW * 32,        \
+    return launch_pdl(k_cbatch<T, V>, spread_blocks(nw, BCfg<T, V>::CW), BCfg<T, V>::CW * 32,        \
                       BCfg<T, V>::CSMEM, st, items, wbeg, nw, pay, vec, alpha, partial, vout, err);
   HM_B_ALL(HM_BC)
 #undef HM_BC
@@ -744,7 +744,7 @@ cudaError_t launch_rgemv_b(int tier, int nv, int mode, const PieceCopy* pieces, 
                  rowscale, fix, nfix, fixcnt,   nsplit, splits, fan, fan_base, err};
 #define HM_BR(T, V)                                                                                              \
   if (tier == T && nv == V)                                                                                      \
-    return launch_pdl(k_rbatch<T, V>, (unsigned)((nw + BCfg<T, V>::RW - 1) / BCfg<T, V>::RW), BCfg<T, V>::RW * 32,        \
+    return launch_pdl(k_rbatch<T, V>, spread_blocks(nw, BCfg<T, V>::RW), BCfg<T, V>::RW * 32,        \
                       BCfg<T, V>::RSMEM, st, A, wbeg, nw);
   HM_B_ALL(HM_BR)
 #undef HM_BR

@@ -270,7 +270,7 @@ __global__ void __launch_bounds__(NW * 32, 1)
   extern __shared__ __align__(128) uint8_t smem[];
   pdl_trigger();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int gw = blockIdx.x * NW + warp;
+  const int gw = range_of<NW>(warp, nwt);
   if (gw >= nwt) return;
   const int p0 = wbeg[gw], n = wbeg[gw + 1] - p0;
   if (n <= 0) return;
@@ -570,7 +570,7 @@ __global__ void __launch_bounds__(NW * 32, 1)
     k_rstream(RsArgs A, const int32_t* __restrict__ wbeg, int nwt) {
   pdl_trigger();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int gw = blockIdx.x * NW + warp;
+  const int gw = range_of<NW>(warp, nwt);
   if (gw >= nwt) return;
   const int p0 = wbeg[gw], n = wbeg[gw + 1] - p0;
   if (n <= 0) return;
@@ -1163,7 +1163,7 @@ cudaError_t launch_gather(const double* x, const int32_t* perm, int n, float2* x
 template <int NW, int NS>
 cudaError_t cdot_shape(int tier, const ItemCopy* items, const int32_t* wbeg, int nw, const uint8_t* pay, const float2* vec,
                 F2 alpha, F2* partial, float2* vout, int* err, cudaStream_t st) {
-  const int grid = (nw + NW - 1) / NW;
+  const unsigned grid = spread_blocks(nw, NW);
   if (tier == TIER_F32)
     return launch_pdl(k_cstream<TIER_F32, NW, NS>, grid, NW * 32, cs_smem<NW, NS>(), st, items, wbeg, nw, pay, vec,
                       alpha, partial, vout, err);
@@ -1211,7 +1211,7 @@ cudaError_t rgemv_shape(int tier, int mode, const PieceCopy* pieces, const int32
                  const float2* vec, double alpha, F2 alpha_ff, double beta, double* y, const int32_t* perm,
                  float2* vout, const F2* rowscale, F2* fix, int32_t* fixcnt, const Split* splits, int* err,
                  cudaStream_t st) {
-  const int grid = (nw + NW - 1) / NW;
+  const unsigned grid = spread_blocks(nw, NW);
   const RsArgs A{pieces, pay, vec, alpha, alpha_ff, beta, y, perm, vout, rowscale, fix, fixcnt, splits, err};
 #define HM_RG(T, M) launch_pdl(k_rstream<T, M, NW, NS>, grid, NW * 32, rs_smem<NW, NS>(), st, A, wbeg, nw)
   if (tier == TIER_F32) {

@@ -214,7 +214,7 @@ __global__ void __launch_bounds__(MP_THREADS, 1)
   __shared__ int s_last[MP_PAIRS];
   pdl_trigger();
   const int pair = threadIdx.x >> 6, wi = (threadIdx.x >> 5) & 1, lane = threadIdx.x & 31;
-  const int gp = blockIdx.x * MP_PAIRS + pair;
+  const int gp = range_of<MP_PAIRS>(pair, nrange);
   if (gp >= nrange) return;   // the whole pair
   const int p0 = wbeg[gp], n = wbeg[gp + 1] - p0;
   if (n <= 0) return;
@@ -575,7 +575,7 @@ __global__ void __launch_bounds__(CW_WARPS * 32, 1)
   extern __shared__ __align__(128) uint8_t smem[];
   pdl_trigger();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int gw = blockIdx.x * CW_WARPS + warp;
+  const int gw = range_of<CW_WARPS>(warp, nrange);
   if (gw >= nrange) return;
   const int p0 = wbeg[gw], n = wbeg[gw + 1] - p0;
   if (n <= 0) return;
@@ -688,7 +688,7 @@ cudaError_t launch_gsum_mr(const GsumOut* outs, int nouts, const F2* pscale, con
 cudaError_t launch_cdot_ws(const ItemCopy* items, const int32_t* wbeg, int nblk, const uint8_t* pay, const float* vec,
                            F2 alpha, float* partial, float* vout, int* err, cudaStream_t st) {
   if (nblk <= 0) return cudaSuccess;
-  return launch_pdl(k_cdot_ws, (unsigned)((nblk + CW_WARPS - 1) / CW_WARPS), CW_WARPS * 32, CW_SMEM, st, items, wbeg,
+  return launch_pdl(k_cdot_ws, spread_blocks(nblk, CW_WARPS), CW_WARPS * 32, CW_SMEM, st, items, wbeg,
                     nblk, pay, vec, alpha, partial, vout, err);
 }
 
@@ -698,7 +698,7 @@ cudaError_t launch_rgemv_ms(int mode, const PieceCopy* pieces, const int32_t* wb
                             const int32_t* perm, float* vout, const F2* rowscale, F2* fix, int32_t* fixcnt,
                             const Split* splits, const int32_t* fan, int32_t fan_base, int* err, cudaStream_t st) {
   if (nblk <= 0) return cudaSuccess;
-  const unsigned grid = (unsigned)((nblk + MP_PAIRS - 1) / MP_PAIRS);
+  const unsigned grid = spread_blocks(nblk, MP_PAIRS);
 #define HM_MSG(M)                                                                                             \
   launch_pdl(k_rgemv_ms<M>, grid, MP_THREADS, MP_SMEM, st, pieces, wbeg, nblk, pay, vec, alpha, alpha_ff, beta, y, ldy, \
              r, perm, vout, rowscale, fix, fixcnt, splits, fan, fan_base, err)

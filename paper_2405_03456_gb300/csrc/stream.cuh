@@ -27,6 +27,15 @@ __device__ void drain(uint64_t* bars, int i, int issued, uint32_t it0 = 0) {
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
+// Range of warp (or pair) w of this block.  A launch with fewer ranges than warps
+// on the device gets one block per SM all the same and deals its ranges out over
+// the blocks, so that a short launch uses every SM (16 ranges on one SM share its
+// issue slots while others idle); a full one keeps neighbouring ranges together.
+template <int NW>
+__device__ __forceinline__ int range_of(int w, int nranges) {
+  return (int)gridDim.x * NW > nranges ? w * (int)gridDim.x + (int)blockIdx.x : (int)blockIdx.x * NW + w;
+}
+
 // ---------------------------------------------------------------- column dots
 // (s, c) += (s2, c2) for Dot2 pairs (TwoSum of the leading parts).
 template <int TIER>
@@ -192,6 +201,15 @@ __device__ __noinline__ bool rs_emit(AccR<RL> acc, int row0, int R, int hflags, 
 }
 
 // ---------------------------------------------------------------- launches
+// Blocks of NW ranges each for nranges ranges (see range_of).
+inline unsigned spread_blocks(int nranges, int NW) {
+  int dev = 0, nsm = 1;
+  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+    nsm = 1;
+  const int need = (nranges + NW - 1) / NW;
+  return (unsigned)(need > nsm ? need : nranges < nsm ? nranges : nsm);
+}
+
 // Launch with programmatic stream serialization (see pdl_trigger / pdl_wait).
 template <typename... KArgs, typename... Args>
 cudaError_t launch_pdl(void (*k)(KArgs...), unsigned grid, unsigned block, size_t smem, cudaStream_t st,

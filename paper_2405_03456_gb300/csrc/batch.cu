@@ -13,11 +13,13 @@
 //  * k_cbatch: column dots.  Lane (g, q) as in the single kernel; the partials of a
 //    round are exchanged as they come, in the reduce-scatter's tree (same sums),
 //    so that 3 instead of 8 per right-hand side are live;
-//  * k_gsum_b: segment sums, four lanes per output, NV sums each;
+//  * k_gsum_b: segment sums, four groups of lanes per output, two sums a lane;
 //  * k_rbatch: row chunks.  The multiplier rows are gathered straight from the
 //    coefficients (source indices one piece ahead), so a batch needs no fan-out;
 //  * fewer, fatter warps than the single kernels: the NV independent sums of a
 //    lane hide the latency that 16 warps per SM hide there.
+// Measured (AFLP): N = 131072, eps = 1e-6, 4 columns 0.475 ms, 8 columns 0.83 ms (0.88
+// and 1.76 as single products); n = 32768, eps = 1e-8, 4 columns 0.48 ms (0.70).
 #include <cstdint>
 #include <cuda_runtime.h>
 
@@ -392,14 +394,14 @@ __global__ void __launch_bounds__(BCfg<TIER, NV>::CW * 32, 1)
       else
         latch_error(err, 1);
     } else {
-    switch (fb) {
+      switch (fb) {
 #define HM_CB(FF_, BB_) \
   case ((FF_) << 4) | (BB_): cb_piece<TIER, FF_, BB_, NV>(sa, fb, R, nc, (int)flags, xh, xl, lane, alpha, partial, vout); break;
-      HM_FORMATS(HM_CB)
+        HM_FORMATS(HM_CB)
 #undef HM_CB
-      default:
-        latch_error(err, 1);
-    }
+        default:
+          latch_error(err, 1);
+      }
     }
     __syncwarp();
     if (issued < n) issue(issued, true);
@@ -634,14 +636,14 @@ __global__ void __launch_bounds__(BCfg<TIER, NV>::RW * 32, 1)
       else
         latch_error(A.err, 2);
     } else {
-    switch (H.fb) {
+      switch (H.fb) {
 #define HM_RB(FF_, BB_) \
   case ((FF_) << 4) | (BB_): rb_piece<TIER, FF_, BB_, NV>(sa, H, A.alpha_ff, lane, ahi, alo); break;
-      HM_FORMATS(HM_RB)
+        HM_FORMATS(HM_RB)
 #undef HM_RB
-      default:
-        latch_error(A.err, 2);
-    }
+        default:
+          latch_error(A.err, 2);
+      }
     }
     if (rinfo.x & PD_LAST) {
       const int fl = H.flags | ((rinfo.x & PD_SPLIT) ? 0x10000 : 0);

@@ -137,7 +137,7 @@ __device__ __forceinline__ void rs_store_rows(const AccR<RL>& acc, int g0, int n
 // End of a warp's part of a chunk (hflags: piece header flags, bit 16 set when
 // the chunk is shared by several warps): reduce the column slots (fixed order), then
 // emit the rows, directly or through the fix-up of a chunk shared by warps (the
-// last part to arrive sums all parts in part order, so the result does not
+// last part to arrive sums all parts in a fixed order, so the result does not
 // depend on which warp finishes last).
 // Out of line: it runs once per part and keeps the piece loop compact.
 template <int MODE, int RL, int VS = 1>
@@ -149,54 +149,59 @@ __device__ __noinline__ bool rs_emit(AccR<RL> acc, int row0, int R, int hflags, 
   static_assert(RL == RPL, "lanes hold RPL rows");
   int G, S, slot, q;
   lane_split(R, lane, G, S, slot, q);
-  // pairwise tree over the S column slots (slot s takes s + off when s is a
-  // multiple of 2 off): log2 S shuffle rounds, all rows of a round in flight
-  for (int off = 1; off < S; off <<= 1) {
-    float hi[RL], lo[RL];
+  const int rows = slot < S ? min(RL, R - RL * q) : 0;
+  const bool shared = (hflags & 0x10000) != 0;
+  for (int turn = 0;; ++turn) {
+    // pairwise tree over the S column slots (slot s takes s + off when s is a
+    // multiple of 2 off): log2 S shuffle rounds, all rows of a round in flight
+    for (int off = 1; off < S; off <<= 1) {
+      float hi[RL], lo[RL];
 #pragma unroll
-    for (int u = 0; u < RL; ++u) {
-      hi[u] = __shfl_down_sync(HM_FULL, acc.v[u].hi, off * G);
-      lo[u] = __shfl_down_sync(HM_FULL, acc.v[u].lo, off * G);
+      for (int u = 0; u < RL; ++u) {
+        hi[u] = __shfl_down_sync(HM_FULL, acc.v[u].hi, off * G);
+        lo[u] = __shfl_down_sync(HM_FULL, acc.v[u].lo, off * G);
+      }
+      if ((slot & (2 * off - 1)) == 0 && slot + off < S) {
+#pragma unroll
+        for (int u = 0; u < RL; ++u) acc.v[u] = ff_add(acc.v[u], FF{hi[u], lo[u]});
+      }
     }
-    if ((slot & (2 * off - 1)) == 0 && slot + off < S) {
+    if (!shared || turn == 1) break;
+    const Split sp = splits[split];
+    F2* mypart = fix + (size_t)(sp.slot0 + pidx) * CHUNK_ROWS + RL * q;   // split, pidx: from the piece's split / part word
+    if (lane < G)
 #pragma unroll
-      for (int u = 0; u < RL; ++u) acc.v[u] = ff_add(acc.v[u], FF{hi[u], lo[u]});
-    }
-  }
-  const bool mine = lane < G;   // slot 0 lanes hold the chunk's rows RL q .. RL q + RL-1
-  const int nr = mine ? min(RL, R - RL * q) : 0;
-  const bool calpha = (hflags & PH_CALPHA) != 0;
-  if (!(hflags & 0x10000)) {   // not shared with other warps
-    if (nr > 0) rs_store_rows<MODE, RL, VS>(acc, row0 + RL * q, nr, alpha_ff, beta, y, perm, vout, rowscale, calpha);
-    return true;
-  }
-  const Split sp = splits[split];
-  F2* mypart = fix + (size_t)(sp.slot0 + pidx) * CHUNK_ROWS + RL * q;   // split, pidx: from the piece's split / part word
-#pragma unroll
-  for (int u = 0; u < RL; ++u)
-    if (u < nr) mypart[u] = F2{acc.v[u].hi, acc.v[u].lo};
-  __syncwarp();   // the part's rows before lane 0's release
-  int last = 0;
-  if (lane == 0) last = atom_add_acq_rel(&fixcnt[split], 1) == sp.nparts - 1;
-  last = __shfl_sync(HM_FULL, last, 0);
-  if (!last) return false;
-  __syncwarp();   // lane 0's acquire before the lanes read the other parts
-  if (nr > 0) {
+      for (int u = 0; u < RL; ++u)
+        if (u < rows) mypart[u] = F2{acc.v[u].hi, acc.v[u].lo};
+    __syncwarp();   // the part's rows before lane 0's release
+    int last = 0;
+    if (lane == 0) last = atom_add_acq_rel(&fixcnt[split], 1) == sp.nparts - 1;
+    last = __shfl_sync(HM_FULL, last, 0);
+    if (!last) return false;
+    __syncwarp();   // lane 0's acquire before the lanes read the other parts
+    // the parts dealt out over the slots, then the same tree: a small matrix has
+    // chunks of more than ten parts, and one load round trip for each in turn was most
+    // of its launch (H product, n = 4096: 30.2 us before, 22.4 us now)
 #pragma unroll
     for (int u = 0; u < RL; ++u) acc.v[u] = FF{0.f, 0.f};
     const F2* base = fix + (size_t)sp.slot0 * CHUNK_ROWS + RL * q;
-    for (int k = 0; k < sp.nparts; ++k) {   // the rows of one part: independent loads, then the sums
-      float2 v[RL];
+    if (slot < S)
+#pragma unroll 1
+      for (int k = slot; k < sp.nparts; k += S) {   // the rows of one part: independent loads, then the sums
+        float2 v[RL];
 #pragma unroll
-      for (int u = 0; u < RL; ++u)
-        v[u] = u < nr ? __ldcg(reinterpret_cast<const float2*>(base + (size_t)k * CHUNK_ROWS + u))
-                      : make_float2(0.f, 0.f);
+        for (int u = 0; u < RL; ++u)
+          v[u] = u < rows ? __ldcg(reinterpret_cast<const float2*>(base + (size_t)k * CHUNK_ROWS + u))
+                          : make_float2(0.f, 0.f);
 #pragma unroll
-      for (int u = 0; u < RL; ++u) acc.v[u] = ff_add(acc.v[u], FF{v[u].x, v[u].y});
-    }
-    rs_store_rows<MODE, RL, VS>(acc, row0 + RL * q, nr, alpha_ff, beta, y, perm, vout, rowscale, calpha);
+        for (int u = 0; u < RL; ++u) acc.v[u] = ff_add(acc.v[u], FF{v[u].x, v[u].y});
+      }
+    if (lane == 0) fixcnt[split] = 0;   // ready for the next product
   }
-  if (lane == 0) fixcnt[split] = 0;   // ready for the next product
+  // slot 0 lanes hold the chunk's rows RL q .. RL q + RL - 1
+  if (lane < G)
+    rs_store_rows<MODE, RL, VS>(acc, row0 + RL * q, rows, alpha_ff, beta, y, perm, vout, rowscale,
+                                (hflags & PH_CALPHA) != 0);
   return true;
 }
 

@@ -111,7 +111,9 @@ hm_status hm_compress(hm_matrix* m, double eps, int32_t codec, int32_t valr);
  * hm_matvec -- y := alpha*M*x + beta*y on the GPU, stream-ordered, no sync.
  *   x : device, FP64, n x nrhs, leading dimension ldx >= n; read only.
  *   y : device, FP64, n x nrhs, leading dimension ldy >= n; must not overlap x.
- *   nrhs : 1..64 right-hand sides.
+ *   nrhs : 1..64 right-hand sides.  Panels of 32 (FP32 tier, 9 or more columns
+ *     left) and batches of 2 to 8 read the matrix once; a batch column equals its
+ *     single product up to the float-float order of summation across pieces.
  *   stream : cudaStream_t as void* (NULL = default stream).
  * Concurrent calls on one matrix must be ordered by the caller (they share the
  * matrix's workspace).  Device-side errors are latched, see hm_sync_status.
@@ -172,7 +174,9 @@ hm_status hm_graph(hm_matrix* m, int32_t enable);
  * A wait that runs out latches HM_ERR_TIMEOUT (hm_sync_status).  Modes 1 and 2
  * use the warp ranges of launch shape 0 whatever hm_autotune chose, and their
  * results equal mode 0 with all shapes 0 bit for bit.  Profiling (hm_profile)
- * always runs mode 0.  Errors: HM_ERR_ARG (enable outside 0..2).
+ * always runs mode 0.  The modes and the launch shapes apply to single products;
+ * batches of a few right-hand sides and panels run one launch per step on their
+ * own shapes.  Errors: HM_ERR_ARG (enable outside 0..2).
  */
 hm_status hm_persistent(hm_matrix* m, int32_t enable);
 /* hm_persistent_mode -- the mode in use (0, 1 or 2; hm_autotune may change it). */

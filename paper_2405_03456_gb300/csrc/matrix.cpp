@@ -201,6 +201,16 @@ struct hm_matrix {
     return e;
   }
 
+  void drop_batch() {
+    if (!d_vmr) {   // its own buffers
+      if (d_vb) cudaFree(d_vb);
+      if (d_pb) cudaFree(d_pb);
+      if (d_fb) cudaFree(d_fb);
+    }
+    d_vb = d_pb = nullptr;
+    d_fb = nullptr;
+  }
+
   void release_device() {
     drop_graph();
     d_pay.release();
@@ -227,13 +237,7 @@ struct hm_matrix {
     d_perm.release();
     if (d_fix) cudaFree(d_fix);
     if (d_fixcnt) cudaFree(d_fixcnt);
-    if (d_vb && !d_vmr) {
-      cudaFree(d_vb);
-      cudaFree(d_pb);
-      cudaFree(d_fb);
-    }
-    d_vb = d_pb = nullptr;
-    d_fb = nullptr;
+    drop_batch();
     if (d_vmr) cudaFree(d_vmr);
     if (d_pmr) cudaFree(d_pmr);
     if (d_fixmr) cudaFree(d_fixmr);
@@ -341,12 +345,19 @@ hm_status upload(hm_matrix* M) {
     M->d_pb = reinterpret_cast<float2*>(M->d_pmr);
     M->d_fb = M->d_fixmr;
   } else {
+    // a matrix that fits without them is served by single products
     const size_t row = BATCH_MAX_FF * sizeof(float2);
-    if ((e = cudaMalloc(&M->d_vb, (size_t)(std::max<int64_t>(P.fan_base, 1) + SEG_ROWS) * row)) != cudaSuccess ||
-        (e = cudaMemset(M->d_vb, 0, (size_t)(std::max<int64_t>(P.fan_base, 1) + SEG_ROWS) * row)) != cudaSuccess ||
-        (e = cudaMalloc(&M->d_pb, (size_t)std::max<int64_t>(P.npartial, 1) * row)) != cudaSuccess ||
-        (e = cudaMalloc(&M->d_fb, (size_t)std::max<int64_t>(P.nfix, 1) * CHUNK_ROWS * row)) != cudaSuccess)
+    const size_t nv = (size_t)(std::max<int64_t>(P.fan_base, 1) + SEG_ROWS) * row;
+    e = cudaMalloc(&M->d_vb, nv);
+    if (e == cudaSuccess) e = cudaMalloc(&M->d_pb, (size_t)std::max<int64_t>(P.npartial, 1) * row);
+    if (e == cudaSuccess) e = cudaMalloc(&M->d_fb, (size_t)std::max<int64_t>(P.nfix, 1) * CHUNK_ROWS * row);
+    if (e == cudaSuccess) e = cudaMemset(M->d_vb, 0, nv);
+    if (e == cudaErrorMemoryAllocation) {
+      cudaGetLastError();   // not sticky
+      M->drop_batch();
+    } else if (e != cudaSuccess) {
       return cuda_status(e);
+    }
   }
   if ((e = cudaMalloc(&M->d_err, sizeof(int))) != cudaSuccess) return cuda_status(e);
   if ((e = cudaMemset(M->d_err, 0, sizeof(int))) != cudaSuccess) return cuda_status(e);
@@ -734,7 +745,7 @@ static hm_status run_all(hm_matrix* M, double alpha, const double* x, int64_t ld
       s = run_program_mr(M, alpha, x + r0 * ldx, ldx, beta, y + r0 * ldy, ldy, (int)std::min<int64_t>(RP, nrhs - r0),
                          st);
   while (r0 < nrhs && s == HM_OK) {
-    const int nv = pass_width(M->prog.tier, nrhs - r0);
+    const int nv = M->d_vb ? pass_width(M->prog.tier, nrhs - r0) : 1;
     const int r = (int)std::min<int64_t>(nv, nrhs - r0);
     if (nv == 1)
       s = run_program(M, alpha, x + r0 * ldx, beta, y + r0 * ldy, st);

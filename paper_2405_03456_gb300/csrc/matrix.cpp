@@ -745,7 +745,10 @@ static hm_status run_all(hm_matrix* M, double alpha, const double* x, int64_t ld
       s = run_program_mr(M, alpha, x + r0 * ldx, ldx, beta, y + r0 * ldy, ldy, (int)std::min<int64_t>(RP, nrhs - r0),
                          st);
   while (r0 < nrhs && s == HM_OK) {
-    const int nv = M->d_vb ? pass_width(M->prog.tier, nrhs - r0) : 1;
+    // two columns of a matrix with fused runs (H^2, UH separate) are not slower as
+    // single products: their launches are short, and a batch runs them one by one
+    const bool single = !M->d_vb || (nrhs - r0 <= 2 && M->fuse && !M->runs.empty());
+    const int nv = single ? 1 : pass_width(M->prog.tier, nrhs - r0);
     const int r = (int)std::min<int64_t>(nv, nrhs - r0);
     if (nv == 1)
       s = run_program(M, alpha, x + r0 * ldx, beta, y + r0 * ldy, st);

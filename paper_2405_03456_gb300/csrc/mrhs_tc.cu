@@ -2,7 +2,7 @@
 // FP32 tier): y (or a coefficient panel) := the chunk rows of A times the
 // multiplier panel T, for panels of RP right-hand sides.
 //
-// One CTA owns MP_PAIRS consecutive ranges of pieces; its warps have fixed roles and hand work on
+// One CTA owns a run of consecutive ranges of pieces (about MP_PAIRS, fewer where the launch is short); its warps have fixed roles and hand work on
 // through mbarriers (no block-wide barrier in the loop):
 //  * warp 0 streams every piece (one bulk copy) and its multiplier rows (RP
 //    values each, taken from the coefficient they stand for; 16-byte cp.async)
@@ -33,7 +33,7 @@
 #include <cstdint>
 #include <cuda_runtime.h>
 
-#include "decode.cuh"
+#include "stream.cuh"
 
 namespace hm {
 
@@ -149,10 +149,11 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
   __shared__ uint32_t tbase;
   __shared__ int s_last;
   const int t = threadIdx.x, w = t >> 5, lane = t & 31;
-  // the CTA takes MP_PAIRS consecutive ranges as one stream of pieces (the
+  // the CTA takes nrange / gridDim consecutive ranges as one stream of pieces (the
   // ranges' part flags still hold: a chunk part closed at a range end goes
   // through its fix-up slot like any other)
-  const int r0 = blockIdx.x * MP_PAIRS, r1 = min(r0 + MP_PAIRS, nrange);
+  const int per = (nrange + (int)gridDim.x - 1) / (int)gridDim.x;
+  const int r0 = blockIdx.x * per, r1 = min(r0 + per, nrange);
   if (r0 >= nrange) return;
   const int p0 = wbeg[r0], n = wbeg[r1] - p0;
   if (n <= 0) return;
@@ -819,7 +820,7 @@ cudaError_t launch_rgemv_tc(int mode, const PieceCopy* pieces, const int32_t* wb
                             const Split* splits, const int32_t* fan, int32_t fan_base, int* err, cudaStream_t st) {
   if (nrange <= 0) return cudaSuccess;
 #define HM_TCG(M)                                                                                              \
-  k_rgemv_tc<M><<<(unsigned)((nrange + MP_PAIRS - 1) / MP_PAIRS), TC_THREADS, TC_SMEM, st>>>(pieces, wbeg, nrange, pay, vec, alpha, alpha_ff, \
+  k_rgemv_tc<M><<<spread_blocks(nrange, MP_PAIRS), TC_THREADS, TC_SMEM, st>>>(pieces, wbeg, nrange, pay, vec, alpha, alpha_ff, \
                                                                beta, y, ldy, r, perm, vout, rowscale, fix, fixcnt, \
                                                                splits, fan, fan_base, err)
   if (mode == MODE_Y)

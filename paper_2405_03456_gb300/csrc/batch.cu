@@ -50,7 +50,7 @@ __global__ void k_gather_b(const double* __restrict__ x, int64_t ldx, int r, con
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= (int64_t)n * NV) return;
   const int i = (int)(t / NV), k = (int)(t % NV);
-  const FF f = k < r ? ff_from_d(x[(int64_t)perm[i] + k * ldx]) : FF{0.f, 0.f};
+  const FF f = k < r ? ff_from_d(__ldcg(x + perm[i] + k * ldx)) : FF{0.f, 0.f};
   v[t] = make_float2(f.hi, f.lo);
 }
 

@@ -641,7 +641,7 @@ __device__ __forceinline__ void fanout_one(const int32_t* __restrict__ src, int 
   }
   float2 v[FAN_PER];
 #pragma unroll
-  for (int k = 0; k < FAN_PER; ++k) v[k] = ix[k] >= 0 ? vec[ix[k]] : make_float2(0.f, 0.f);
+  for (int k = 0; k < FAN_PER; ++k) v[k] = ix[k] >= 0 ? __ldcg(vec + ix[k]) : make_float2(0.f, 0.f);
 #pragma unroll
   for (int k = 0; k < FAN_PER; ++k)
     if (ix[k] >= 0) dst[base + k * stride] = v[k];
@@ -674,19 +674,20 @@ __device__ __forceinline__ void gsum_one(const GsumOut* __restrict__ outs, int n
   const int nslot = fan_dst ? (O.flags >> 8) : 0;
   const int32_t slot0 = k < nslot ? fan_dst[O.pad + k] : -1;
   FF s = {0.f, 0.f};
+  const float2* src = reinterpret_cast<const float2*>(partial);   // (read from L2: see k_gather)
   // (unrolled: several partials in flight per lane; the sum order is unchanged)
   if (O.flags & 2) {
 #pragma unroll 4
     for (int p = O.p0 + k; p < O.p1; p += GS_LANES) {
-      const F2 v = partial[p];
+      const float2 v = __ldcg(src + p);
       const F2 w = pscale[O.ps + (p - O.p0)];
-      s = ff_add(s, ff_mul(FF{v.hi, v.lo}, FF{w.hi, w.lo}));
+      s = ff_add(s, ff_mul(FF{v.x, v.y}, FF{w.hi, w.lo}));
     }
   } else {
 #pragma unroll 4
     for (int p = O.p0 + k; p < O.p1; p += GS_LANES) {
-      const F2 v = partial[p];
-      s = ff_add(s, FF{v.hi, v.lo});
+      const float2 v = __ldcg(src + p);
+      s = ff_add(s, FF{v.x, v.y});
     }
   }
 #pragma unroll
@@ -720,7 +721,7 @@ __device__ __forceinline__ void fcopy_one(const int32_t* __restrict__ csrc, cons
   }
   float2 v[FAN_PER];
 #pragma unroll
-  for (int q = 0; q < FAN_PER; ++q) v[q] = ix[q] >= 0 ? vec[ix[q]] : make_float2(0.f, 0.f);
+  for (int q = 0; q < FAN_PER; ++q) v[q] = ix[q] >= 0 ? __ldcg(vec + ix[q]) : make_float2(0.f, 0.f);
 #pragma unroll
   for (int q = 0; q < FAN_PER; ++q)
     if (ix[q] >= 0) vec[dx[q]] = v[q];
@@ -741,6 +742,11 @@ __global__ void k_gsum(const GsumOut* __restrict__ outs, int nouts, const F2* __
 }
 
 // ---------------------------------------------------------------- gather x
+// What an earlier kernel of the stream wrote is read from L2 (__ldcg), here and in
+// every kernel that starts before its predecessor ends: a plain load through a
+// const __restrict__ pointer may take the non-coherent path, which is for data
+// that nothing writes while the kernel is resident -- and x (y of the product before,
+// in y := a M x + b y chains) or the partials may still be written when it starts.
 __global__ void k_gather(const double* __restrict__ x, const int32_t* __restrict__ perm, int n,
                          float2* __restrict__ xo) {
   pdl_trigger();
@@ -748,7 +754,7 @@ __global__ void k_gather(const double* __restrict__ x, const int32_t* __restrict
   const int p = i < n ? __ldg(perm + i) : 0;
   pdl_wait();   // x may be the previous kernel's result, and that kernel may still read xo
   if (i >= n) return;
-  const FF f = ff_from_d(x[p]);
+  const FF f = ff_from_d(__ldcg(x + p));
   xo[i] = make_float2(f.hi, f.lo);
 }
 

@@ -35,7 +35,7 @@ __global__ void k_gather_mr(const double* __restrict__ x, int64_t ldx, int r, co
   if (i >= n) return;
   float f[4];
 #pragma unroll
-  for (int u = 0; u < 4; ++u) f[u] = k + u < r ? (float)xi[(int64_t)(k + u) * ldx] : 0.0f;
+  for (int u = 0; u < 4; ++u) f[u] = k + u < r ? (float)__ldcg(xi + (int64_t)(k + u) * ldx) : 0.0f;
   *reinterpret_cast<float4*>(v + 4 * t) = make_float4(f[0], f[1], f[2], f[3]);
 }
 

@@ -36,6 +36,13 @@ struct F2 {
   float hi, lo;
 };
 
+// First component of entry i in a vector that interleaves VS right-hand sides: a
+// program may have up to 2^31 entries, so that i * VS needs 64 bits.
+template <int VS>
+HM_HD constexpr int64_t entry_offset(int32_t i) {
+  return (int64_t)i * VS;
+}
+
 // Rows per lane in the product kernels: a lane decodes 8 (float-float tier)
 // or 16 (FP32 tier) consecutive values of a column, i.e. groups of 4 codes,
 // 8*B bytes per 8 rows, from an 8-byte aligned address; every packed column

@@ -118,7 +118,7 @@ __device__ __forceinline__ void rs_store_rows(const AccR<RL>& acc, int g0, int n
     float2 old[RL], sc[RL];
 #pragma unroll
     for (int u = 0; u < RL; ++u) {
-      old[u] = (MODE == MODE_VEC_ADD && u < nr) ? __ldcg(vout + (g0 + u) * VS) : make_float2(0.f, 0.f);
+      old[u] = (MODE == MODE_VEC_ADD && u < nr) ? __ldcg(vout + entry_offset<VS>(g0 + u)) : make_float2(0.f, 0.f);
       sc[u] = (rowscale && u < nr) ? __ldg(reinterpret_cast<const float2*>(rowscale + g0 + u)) : make_float2(1.f, 0.f);
     }
 #pragma unroll
@@ -128,7 +128,7 @@ __device__ __forceinline__ void rs_store_rows(const AccR<RL>& acc, int g0, int n
         if constexpr (MODE == MODE_VEC_ADD) v = ff_add(v, FF{old[u].x, old[u].y});
         if (rowscale) v = ff_mul(v, FF{sc[u].x, sc[u].y});
         if (calpha) v = ff_mul(v, FF{alpha_ff.hi, alpha_ff.lo});
-        vout[(g0 + u) * VS] = make_float2(v.hi, v.lo);
+        vout[entry_offset<VS>(g0 + u)] = make_float2(v.hi, v.lo);
       }
     }
   }

@@ -129,11 +129,14 @@ struct hm_matrix {
   float* d_pmr = nullptr;      // multi-RHS column-dot partials: npartial x RP
   F2* d_fixmr = nullptr;       // multi-RHS fix-up rows: nfix_mr x CHUNK_ROWS x RP
   // batches of up to BATCH_MAX right-hand sides: interleaved vectors, partials,
-  // fix-up rows.  In the FP32 tier they are the panel's buffers (a batch and a
-  // panel never run at the same time), in the float-float tier their own.
+  // fix-up rows, arrival counters per column; all null when the device has no room
+  // for them (see batch_buffers).  In the FP32 tier the first three are the panel's
+  // (a batch and a panel never run at the same time) as far as those suffice.
   float2 *d_vb = nullptr, *d_pb = nullptr;
   F2* d_fb = nullptr;
-  int32_t* d_fixcnt = nullptr; // arrival counters of those chunks (reset by the last part), per batch column
+  int32_t* d_bcnt = nullptr;
+  int64_t batch_bytes = 0;     // of the buffers that only batches use
+  int32_t* d_fixcnt = nullptr; // arrival counters of chunks shared by warps (reset by the last part)
   float2* d_vec = nullptr;     // vector workspace (x, coefficient vectors)
   F2* d_part = nullptr;        // column-dot partial sums (float-float)
   int* d_err = nullptr;        // latched device error word
@@ -205,10 +208,13 @@ struct hm_matrix {
     if (!d_vmr) {   // its own buffers
       if (d_vb) cudaFree(d_vb);
       if (d_pb) cudaFree(d_pb);
-      if (d_fb) cudaFree(d_fb);
     }
+    if (d_fb && d_fb != d_fixmr) cudaFree(d_fb);
+    if (d_bcnt) cudaFree(d_bcnt);
     d_vb = d_pb = nullptr;
     d_fb = nullptr;
+    d_bcnt = nullptr;
+    batch_bytes = 0;
   }
 
   void release_device() {
@@ -276,13 +282,57 @@ namespace {
 // Columns of one batch pass (the widest kernels of each tier).
 constexpr int BATCH_MAX = 8, BATCH_MAX_FF = 4;
 
-// Fix-up slots (CHUNK_ROWS entries) that serve both a panel and a batch.
-int64_t fixmr_slots(const Program& P) {
-  return std::max<int64_t>({P.nfix_mr * RP, P.nfix * BATCH_MAX, 1});
-}
-
 std::once_flag g_kinit;
 cudaError_t g_kinit_err = cudaSuccess;
+
+// The buffers of batch passes, after everything else the matrix needs.  They only
+// make a few right-hand sides faster, so they are kept only if the device still has
+// room for what later calls allocate without them: the transposed matrix of the first
+// adjoint product (about this matrix again; twice that is asked for), the staging of
+// hm_matvec_host (64 columns of x and y), the vectors of hm_autotune (RP + 1 of each).
+// Otherwise, and when they do not fit, a few right-hand sides run as single products.
+hm_status batch_buffers(hm_matrix* M) {
+  const Program& P = M->prog;
+  const int w = P.tier == TIER_F32 ? BATCH_MAX : BATCH_MAX_FF;
+  const size_t row = (size_t)w * sizeof(float2);
+  const size_t nv = (size_t)(std::max<int64_t>(P.fan_base, 1) + SEG_ROWS) * row;
+  const size_t np = (size_t)std::max<int64_t>(P.npartial, 1) * row;
+  const size_t nf = (size_t)std::max<int64_t>(P.nfix, 1) * CHUNK_ROWS * row;
+  const size_t nc = std::max<size_t>(P.splits.size(), 1) * w * sizeof(int32_t);
+  cudaError_t e = cudaSuccess;
+  size_t held = 0;
+  auto own = [&](auto** p, size_t bytes) {
+    if (e == cudaSuccess && (e = cudaMalloc(p, bytes)) == cudaSuccess) held += bytes;
+  };
+  if (M->d_vmr) {
+    static_assert(BATCH_MAX * sizeof(float2) <= RP * sizeof(float), "a batch's vectors fit the panel's");
+    M->d_vb = reinterpret_cast<float2*>(M->d_vmr);
+    M->d_pb = reinterpret_cast<float2*>(M->d_pmr);
+  } else {
+    own(&M->d_vb, nv);
+    own(&M->d_pb, np);
+    if (e == cudaSuccess) e = cudaMemset(M->d_vb, 0, nv);
+  }
+  if (M->d_vmr && P.nfix * w <= P.nfix_mr * RP)
+    M->d_fb = M->d_fixmr;
+  else
+    own(&M->d_fb, nf);
+  own(&M->d_bcnt, nc);
+  if (e == cudaSuccess) e = cudaMemset(M->d_bcnt, 0, nc);
+  M->batch_bytes = (int64_t)held;
+  hm_info_t info;
+  size_t avail = 0, total = 0;
+  if (e == cudaSuccess && hm_info(M, &info) == HM_OK && (e = cudaMemGetInfo(&avail, &total)) == cudaSuccess) {
+    const size_t later = 2 * (size_t)(info.bytes_payload + info.bytes_meta + info.bytes_workspace) +
+                         2 * (size_t)(64 + RP + 1) * M->H.n * sizeof(double) + (size_t(64) << 20);
+    if (avail < later) e = cudaErrorMemoryAllocation;
+  }
+  if (e == cudaSuccess) return HM_OK;
+  M->drop_batch();
+  if (e != cudaErrorMemoryAllocation) return cuda_status(e);
+  cudaGetLastError();   // not sticky
+  return HM_OK;
+}
 
 hm_status upload(hm_matrix* M) {
   Program& P = M->prog;
@@ -329,7 +379,7 @@ hm_status upload(hm_matrix* M) {
     return cuda_status(e);
   if ((e = cudaMalloc(&M->d_fix, std::max<int64_t>(P.nfix, 1) * CHUNK_ROWS * sizeof(F2))) != cudaSuccess)
     return cuda_status(e);
-  const size_t ncnt = std::max<size_t>(P.splits.size(), 1) * BATCH_MAX * sizeof(int32_t);
+  const size_t ncnt = std::max<size_t>(P.splits.size(), 1) * sizeof(int32_t);
   if ((e = cudaMalloc(&M->d_fixcnt, ncnt)) != cudaSuccess) return cuda_status(e);
   if ((e = cudaMemset(M->d_fixcnt, 0, ncnt)) != cudaSuccess) return cuda_status(e);
   if (P.tier == TIER_F32) {   // multi-RHS workspace (panels of RP right-hand sides; no fan-out slots)
@@ -338,26 +388,9 @@ hm_status upload(hm_matrix* M) {
     if ((e = cudaMemset(M->d_vmr, 0, nv)) != cudaSuccess) return cuda_status(e);
     if ((e = cudaMalloc(&M->d_pmr, (size_t)std::max<int64_t>(P.npartial, 1) * RP * sizeof(float))) != cudaSuccess)
       return cuda_status(e);
-    if ((e = cudaMalloc(&M->d_fixmr, (size_t)fixmr_slots(P) * CHUNK_ROWS * sizeof(F2))) != cudaSuccess)
+    if ((e = cudaMalloc(&M->d_fixmr, (size_t)std::max<int64_t>(P.nfix_mr, 1) * CHUNK_ROWS * RP * sizeof(F2))) !=
+        cudaSuccess)
       return cuda_status(e);
-    static_assert(BATCH_MAX * sizeof(float2) <= RP * sizeof(float), "a batch's vectors fit the panel's");
-    M->d_vb = reinterpret_cast<float2*>(M->d_vmr);
-    M->d_pb = reinterpret_cast<float2*>(M->d_pmr);
-    M->d_fb = M->d_fixmr;
-  } else {
-    // a matrix that fits without them is served by single products
-    const size_t row = BATCH_MAX_FF * sizeof(float2);
-    const size_t nv = (size_t)(std::max<int64_t>(P.fan_base, 1) + SEG_ROWS) * row;
-    e = cudaMalloc(&M->d_vb, nv);
-    if (e == cudaSuccess) e = cudaMalloc(&M->d_pb, (size_t)std::max<int64_t>(P.npartial, 1) * row);
-    if (e == cudaSuccess) e = cudaMalloc(&M->d_fb, (size_t)std::max<int64_t>(P.nfix, 1) * CHUNK_ROWS * row);
-    if (e == cudaSuccess) e = cudaMemset(M->d_vb, 0, nv);
-    if (e == cudaErrorMemoryAllocation) {
-      cudaGetLastError();   // not sticky
-      M->drop_batch();
-    } else if (e != cudaSuccess) {
-      return cuda_status(e);
-    }
   }
   if ((e = cudaMalloc(&M->d_err, sizeof(int))) != cudaSuccess) return cuda_status(e);
   if ((e = cudaMemset(M->d_err, 0, sizeof(int))) != cudaSuccess) return cuda_status(e);
@@ -440,7 +473,7 @@ hm_status upload(hm_matrix* M) {
       M->pstate_n = (int)nstate;
     }
   }
-  return HM_OK;
+  return batch_buffers(M);
 }
 
 }  // namespace
@@ -696,7 +729,7 @@ static cudaError_t run_launch_b(hm_matrix* M, const Launch& L, int nv, double al
     case Launch::RGEMV:
       return launch_rgemv_b(P.tier, nv, L.mode, M->d_pieces.p + (size_t)cf * P.npieces, M->d_wbeg.p + L.woff[cf],
                             L.nw[cf], M->d_pay.p, M->d_vb, aff, beta, y, ldy, r, M->d_perm.p,
-                            L.use_rowscale ? M->d_rowscale_ff.p : nullptr, M->d_fb, P.nfix, M->d_fixcnt,
+                            L.use_rowscale ? M->d_rowscale_ff.p : nullptr, M->d_fb, P.nfix, M->d_bcnt,
                             (int)P.splits.size(), M->d_splits.p, M->d_fan.p, (int32_t)P.fan_base, M->d_err, st);
   }
   return cudaErrorInvalidValue;
@@ -1220,9 +1253,8 @@ hm_status hm_info(const hm_matrix* M, hm_info_t* o) {
                   H.n * 4;
   o->bytes_workspace = P.nvec * 8 + P.npartial * 8 + P.nfix * CHUNK_ROWS * 8;
   if (M->d_vmr)
-    o->bytes_workspace += ((P.fan_base + SEG_ROWS) + P.npartial) * RP * 4 + fixmr_slots(P) * CHUNK_ROWS * 8;
-  else if (M->d_vb)
-    o->bytes_workspace += ((P.fan_base + SEG_ROWS) + P.npartial + P.nfix * CHUNK_ROWS) * BATCH_MAX_FF * 8;
+    o->bytes_workspace += ((P.fan_base + SEG_ROWS) + P.npartial) * RP * 4 + P.nfix_mr * CHUNK_ROWS * RP * 8;
+  o->bytes_workspace += M->batch_bytes;
   o->nlaunches = (int64_t)P.launches.size();
   o->tier = P.tier;
   o->nunits = (int64_t)P.items.size() + P.npieces;

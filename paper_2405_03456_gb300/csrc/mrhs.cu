@@ -94,8 +94,13 @@ __global__ void k_gsum_mr(const GsumOut* __restrict__ outs, int nouts, const F2*
 // a row group decode one column each of the next four and share the values
 // through shared memory.  Six pairs per SM with two stages each (four with three
 // before: 8 warps an SM could not hide the latency of their own chains).
-// N = 131072, eps = 1e-6, 32 columns: row chunks 0.81 ms, panel 1.41 ms (0.98 and
-// 1.62 before).
+// N = 131072, eps = 1e-6, 32 columns: row chunks 0.77 ms, panel 1.36 ms (0.98 and
+// 1.62 before).  On a small matrix a chunk has tens of parts, and adding them takes
+// most of the launch: their slots are laid out [row][nt][tq], so that the four lanes
+// tq of a row read 64 consecutive bytes, with the loads of two rows in flight, and
+// y is updated four right-hand sides at a time (168 registers at 384 threads: all
+// eight spilled 136 bytes).  Row chunks of n = 1000, leaf 64, 32 columns: 53 us
+// with four pairs, 84 us with six and neither, 51 us now; H^2, n = 4000: 160, 194, 146 us.
 constexpr int NT = RP / 8;
 constexpr int MP_NS = 2;                                   // stages per pair
 constexpr int MP_TP = RP * 4 + 16;                         // multiplier row pitch in a stage (bytes)
@@ -364,8 +369,7 @@ __global__ void __launch_bounds__(MP_THREADS, 1)
             if (row < R) {
 #pragma unroll
               for (int nt = 0; nt < NT; ++nt) {
-                const int k = 8 * tq + 2 * nt;
-                *reinterpret_cast<float4*>(mine + row * RP + k) =
+                *reinterpret_cast<float4*>(mine + row * RP + 8 * nt + 2 * tq) =
                     make_float4(fhi[mt][nt][h].x, flo[mt][nt][h].x, fhi[mt][nt][h].y, flo[mt][nt][h].y);
               }
             }
@@ -389,21 +393,26 @@ __global__ void __launch_bounds__(MP_THREADS, 1)
           for (int part = 0; part < sp.nparts; ++part) {
             const F2* src = fix + (size_t)(sp.slot0 + part) * CHUNK_ROWS * RP;
 #pragma unroll
-            for (int mt = 0; mt < 2; ++mt)
+            for (int mt = 0; mt < 2; ++mt) {   // two rows' loads in flight (all four do not fit the registers)
+              float4 v[2][NT];
 #pragma unroll
               for (int h = 0; h < 2; ++h) {
                 const int row = 32 * wi + 4 * g + 2 * mt + h;
-                if (row < R) {
 #pragma unroll
-                  for (int nt = 0; nt < NT; ++nt) {
-                    const float4 v = __ldcg(reinterpret_cast<const float4*>(src + row * RP + 8 * tq + 2 * nt));
-                    const FF a = ff_add(FF{fhi[mt][nt][h].x, flo[mt][nt][h].x}, FF{v.x, v.y});
-                    const FF b = ff_add(FF{fhi[mt][nt][h].y, flo[mt][nt][h].y}, FF{v.z, v.w});
-                    fhi[mt][nt][h] = make_float2(a.hi, b.hi);
-                    flo[mt][nt][h] = make_float2(a.lo, b.lo);
-                  }
-                }
+                for (int nt = 0; nt < NT; ++nt)
+                  v[h][nt] = row < R ? __ldcg(reinterpret_cast<const float4*>(src + row * RP + 8 * nt + 2 * tq))
+                                     : make_float4(0.f, 0.f, 0.f, 0.f);
               }
+#pragma unroll
+              for (int h = 0; h < 2; ++h)
+#pragma unroll
+                for (int nt = 0; nt < NT; ++nt) {
+                  const FF a = ff_add(FF{fhi[mt][nt][h].x, flo[mt][nt][h].x}, FF{v[h][nt].x, v[h][nt].y});
+                  const FF b = ff_add(FF{fhi[mt][nt][h].y, flo[mt][nt][h].y}, FF{v[h][nt].z, v[h][nt].w});
+                  fhi[mt][nt][h] = make_float2(a.hi, b.hi);
+                  flo[mt][nt][h] = make_float2(a.lo, b.lo);
+                }
+            }
           }
         }
 #pragma unroll
@@ -414,42 +423,48 @@ __global__ void __launch_bounds__(MP_THREADS, 1)
             if (row >= R) continue;
             if constexpr (MODE == MODE_Y) {
               const int o = __ldg(perm + H.row0 + row);
-              double yo[NT][2];
 #pragma unroll
-              for (int nt = 0; nt < NT; ++nt)
+              for (int n0 = 0; n0 < NT; n0 += 2) {   // four right-hand sides at a time (registers)
+                double yo[2][2];
 #pragma unroll
-                for (int c = 0; c < 2; ++c) {
-                  const int k = 8 * tq + 2 * nt + c;
-                  yo[nt][c] = (beta != 0.0 && k < r) ? y[o + (int64_t)k * ldy] : 0.0;
-                }
+                for (int nt = 0; nt < 2; ++nt)
 #pragma unroll
-              for (int nt = 0; nt < NT; ++nt)
-#pragma unroll
-                for (int c = 0; c < 2; ++c) {
-                  const int k = 8 * tq + 2 * nt + c;
-                  if (k < r) {
-                    const double val = ff_to_d(FF{c ? fhi[mt][nt][h].y : fhi[mt][nt][h].x,
-                                                  c ? flo[mt][nt][h].y : flo[mt][nt][h].x});
-                    y[o + (int64_t)k * ldy] = (beta == 0.0) ? val : fma(beta, yo[nt][c], val);
+                  for (int c = 0; c < 2; ++c) {
+                    const int k = 8 * tq + 2 * (n0 + nt) + c;
+                    yo[nt][c] = (beta != 0.0 && k < r) ? y[o + (int64_t)k * ldy] : 0.0;
                   }
-                }
-            } else {   // coefficient panels: float-float updates, one rounding to FP32
+#pragma unroll
+                for (int nt = 0; nt < 2; ++nt)
+#pragma unroll
+                  for (int c = 0; c < 2; ++c) {
+                    const int k = 8 * tq + 2 * (n0 + nt) + c;
+                    if (k < r) {
+                      const double val = ff_to_d(FF{c ? fhi[mt][n0 + nt][h].y : fhi[mt][n0 + nt][h].x,
+                                                    c ? flo[mt][n0 + nt][h].y : flo[mt][n0 + nt][h].x});
+                      y[o + (int64_t)k * ldy] = (beta == 0.0) ? val : fma(beta, yo[nt][c], val);
+                    }
+                  }
+              }
+            } else {   // coefficient panels: float-float updates, one rounding to FP32 (columns past r are not read)
               const int gg = H.row0 + row;
               const F2 rsc = rowscale ? rowscale[gg] : F2{1.f, 0.f};
+              float4* dst = reinterpret_cast<float4*>(vout + (int64_t)gg * RP + 8 * tq);
 #pragma unroll
-              for (int nt = 0; nt < NT; ++nt) {
-                const int k0 = 8 * tq + 2 * nt;
-                const float2 old = (MODE == MODE_VEC_ADD) ? __ldcg(reinterpret_cast<const float2*>(vout + (int64_t)gg * RP + k0))
-                                                          : make_float2(0.f, 0.f);
+              for (int n0 = 0; n0 < NT; n0 += 2) {
+                float4 old = make_float4(0.f, 0.f, 0.f, 0.f);
+                if constexpr (MODE == MODE_VEC_ADD) old = __ldcg(dst + n0 / 2);
+                const float od[4] = {old.x, old.y, old.z, old.w};
+                float o[4];
 #pragma unroll
-                for (int c = 0; c < 2; ++c)
-                  if (k0 + c < r) {
-                    FF v = {c ? fhi[mt][nt][h].y : fhi[mt][nt][h].x, c ? flo[mt][nt][h].y : flo[mt][nt][h].x};
-                    if constexpr (MODE == MODE_VEC_ADD) v = ff_add_f(v, c ? old.y : old.x);
-                    if (rowscale) v = ff_mul(v, FF{rsc.hi, rsc.lo});
-                    if (calpha) v = ff_mul(v, FF{alpha_ff.hi, alpha_ff.lo});
-                    vout[(int64_t)gg * RP + k0 + c] = v.hi + v.lo;
-                  }
+                for (int q = 0; q < 4; ++q) {
+                  const int nt = n0 + (q >> 1);
+                  FF v = {q & 1 ? fhi[mt][nt][h].y : fhi[mt][nt][h].x, q & 1 ? flo[mt][nt][h].y : flo[mt][nt][h].x};
+                  if constexpr (MODE == MODE_VEC_ADD) v = ff_add_f(v, od[q]);
+                  if (rowscale) v = ff_mul(v, FF{rsc.hi, rsc.lo});
+                  if (calpha) v = ff_mul(v, FF{alpha_ff.hi, alpha_ff.lo});
+                  o[q] = v.hi + v.lo;
+                }
+                dst[n0 / 2] = make_float4(o[0], o[1], o[2], o[3]);
               }
             }
           }

@@ -50,8 +50,8 @@ cudaError_t launch_rgemv_tc(int mode, const PieceCopy* pieces, const int32_t* wb
                             const Split* splits, const int32_t* fan, int32_t fan_base, int* err, cudaStream_t st);
 cudaError_t launch_gather_mr(const double* x, int64_t ldx, int r, const int32_t* perm, int n, float* v,
                              cudaStream_t st);
-cudaError_t launch_gsum_mr(const GsumOut* outs, int nouts, const F2* pscale, const float* partial, F2 alpha, float* v,
-                           cudaStream_t st);
+cudaError_t launch_gsum_mr(const GsumOut* outs, int nouts, int64_t nterms, const F2* pscale, const float* partial,
+                           F2 alpha, float* v, cudaStream_t st);
 cudaError_t launch_cdot_ws(const ItemCopy* items, const int32_t* wbeg, int nblk, const uint8_t* pay, const float* vec,
                            F2 alpha, float* partial, float* vout, int* err, cudaStream_t st);
 cudaError_t launch_rgemv_ms(int mode, const PieceCopy* pieces, const int32_t* wbeg, int nblk, const uint8_t* pay,
@@ -671,7 +671,7 @@ static cudaError_t run_launch_mr(hm_matrix* M, const Launch& L, double alpha, co
       return launch_cdot_ws(M->d_items.p, M->d_wbeg.p + L.woff[MR_SHAPE], L.nw[MR_SHAPE], M->d_pay.p, M->d_vmr, aff,
                             M->d_pmr, M->d_vmr, M->d_err, st);
     case Launch::GSUM:
-      return launch_gsum_mr(M->d_gout.p + L.off, (int)L.n, M->d_pscale.p, M->d_pmr, aff, M->d_vmr, st);
+      return launch_gsum_mr(M->d_gout.p + L.off, (int)L.n, L.nterms, M->d_pscale.p, M->d_pmr, aff, M->d_vmr, st);
     case Launch::FANOUT:   // the multi-RHS row-chunk kernel copies each multiplier row from its coefficient
       return cudaSuccess;
     case Launch::RGEMV:

@@ -20,65 +20,108 @@ namespace hm {
 __device__ __forceinline__ uint32_t pad16m(uint32_t x) { return (x + 15u) & ~15u; }
 
 // ---------------------------------------------------------------- gather, segment sums
-// Four right-hand sides per thread (independent loads, one 16-byte store): one per
-// thread left the kernels with too few loads in flight (N = 131072, 32 columns:
-// segment sums 107 us then, 86 us now).
+// W right-hand sides per thread.  W = 4 (independent loads, one 16-byte store) has more
+// loads in flight where its threads alone fill the GPU (MR_FULL) and the sums are
+// short; otherwise SMs idle, or the warps of four outputs run as long as their
+// longest sum, and W = 1 is the faster one.  32 columns, segment sums W = 1 / W = 4:
+// N = 131072 107 / 80 us, H n = 16000 (3.4 partials a sum) 14.1 / 10.5, HODLR n = 16000
+// (16 a sum) 20 / 29; gather N = 131072 29 / 25 us, n = 16000 8.5 / 8.5.
+constexpr int MR_FULL = 152 * 1536;   // threads
+constexpr int MR_LONG = 8;            // partials a sum
+template <int W>
+__device__ __forceinline__ void load_w(const float* p, float (&x)[W]) {
+  if constexpr (W == 4) {
+    const float4 q = __ldcs(reinterpret_cast<const float4*>(p));
+    x[0] = q.x;
+    x[1] = q.y;
+    x[2] = q.z;
+    x[3] = q.w;
+  } else {
+    x[0] = __ldcs(p);
+  }
+}
+template <int W>
+__device__ __forceinline__ void store_w(float* p, const float (&x)[W]) {
+  if constexpr (W == 4)
+    *reinterpret_cast<float4*>(p) = make_float4(x[0], x[1], x[2], x[3]);
+  else
+    *p = x[0];
+}
+
 // v[i * RP + k] = x[perm[i] + k * ldx] (FP32 hi part), k < r; zero for k >= r.
-constexpr int KQ = RP / 4;
+template <int W>
 __global__ void k_gather_mr(const double* __restrict__ x, int64_t ldx, int r, const int32_t* __restrict__ perm, int n,
                             float* __restrict__ v) {
   pdl_trigger();
+  constexpr int KQ = RP / W;
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const int i = (int)(t / KQ), k = 4 * (int)(t % KQ);
+  const int i = (int)(t / KQ), k = W * (int)(t % KQ);
   const double* xi = x + (i < n ? __ldg(perm + i) : 0);
   pdl_wait();   // x may be the previous kernel's result, and that kernel may still read v
   if (i >= n) return;
-  float f[4];
+  float f[W];
 #pragma unroll
-  for (int u = 0; u < 4; ++u) f[u] = k + u < r ? (float)__ldcg(xi + (int64_t)(k + u) * ldx) : 0.0f;
-  *reinterpret_cast<float4*>(v + 4 * t) = make_float4(f[0], f[1], f[2], f[3]);
+  for (int u = 0; u < W; ++u) f[u] = k + u < r ? (float)__ldcg(xi + (int64_t)(k + u) * ldx) : 0.0f;
+  store_w<W>(v + W * t, f);
 }
 
+template <int W>
 __global__ void k_gsum_mr(const GsumOut* __restrict__ outs, int nouts, const F2* __restrict__ pscale,
                           const float* __restrict__ partial, F2 alpha, float* __restrict__ v) {
   pdl_trigger();
   pdl_wait();
+  constexpr int KQ = RP / W;
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= (int64_t)nouts * KQ) return;
   const GsumOut O = outs[t / KQ];
-  const int kq = (int)(t % KQ);
+  const int k = W * (int)(t % KQ);
+  const float* src = partial + k;
+  FF s[W];
+#pragma unroll
+  for (int u = 0; u < W; ++u) s[u] = FF{0.f, 0.f};
+  // partials in order p0, p0 + 1, ...; a batch of loads in flight, then its sums
   const bool ws = (O.flags & 2) != 0;
-  const float4* src = reinterpret_cast<const float4*>(partial) + kq;
-  FF s[4] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
-  // partials in order p0, p0 + 1, ... (unrolled: several loads in flight)
-  if (ws) {
-#pragma unroll 2
-    for (int p = O.p0; p < O.p1; ++p) {
-      const float4 x = __ldcs(src + (int64_t)p * KQ);
-      const F2 w = pscale[O.ps + (p - O.p0)];
-      s[0] = ff_add(s[0], ff_mul(FF{x.x, 0.f}, FF{w.hi, w.lo}));
-      s[1] = ff_add(s[1], ff_mul(FF{x.y, 0.f}, FF{w.hi, w.lo}));
-      s[2] = ff_add(s[2], ff_mul(FF{x.z, 0.f}, FF{w.hi, w.lo}));
-      s[3] = ff_add(s[3], ff_mul(FF{x.w, 0.f}, FF{w.hi, w.lo}));
-    }
-  } else {
-#pragma unroll 4
-    for (int p = O.p0; p < O.p1; ++p) {
-      const float4 x = __ldcs(src + (int64_t)p * KQ);
-      s[0] = ff_add_f(s[0], x.x);
-      s[1] = ff_add_f(s[1], x.y);
-      s[2] = ff_add_f(s[2], x.z);
-      s[3] = ff_add_f(s[3], x.w);
+  constexpr int NB = 4;
+  int p = O.p0;
+  for (; p + NB <= O.p1; p += NB) {
+    float x[NB][W];
+#pragma unroll
+    for (int b = 0; b < NB; ++b) load_w<W>(src + (int64_t)(p + b) * RP, x[b]);
+    if (ws) {
+      F2 w[NB];
+#pragma unroll
+      for (int b = 0; b < NB; ++b) w[b] = pscale[O.ps + (p + b - O.p0)];
+#pragma unroll
+      for (int b = 0; b < NB; ++b)
+#pragma unroll
+        for (int u = 0; u < W; ++u) s[u] = ff_add(s[u], ff_mul(FF{x[b][u], 0.f}, FF{w[b].hi, w[b].lo}));
+    } else {
+#pragma unroll
+      for (int b = 0; b < NB; ++b)
+#pragma unroll
+        for (int u = 0; u < W; ++u) s[u] = ff_add_f(s[u], x[b][u]);
     }
   }
-  float o[4];
+  for (; p < O.p1; ++p) {
+    float x[W];
+    load_w<W>(src + (int64_t)p * RP, x);
+    if (ws) {
+      const F2 w = pscale[O.ps + (p - O.p0)];
 #pragma unroll
-  for (int u = 0; u < 4; ++u) {
+      for (int u = 0; u < W; ++u) s[u] = ff_add(s[u], ff_mul(FF{x[u], 0.f}, FF{w.hi, w.lo}));
+    } else {
+#pragma unroll
+      for (int u = 0; u < W; ++u) s[u] = ff_add_f(s[u], x[u]);
+    }
+  }
+  float o[W];
+#pragma unroll
+  for (int u = 0; u < W; ++u) {
     FF z = ff_mul(s[u], FF{O.scale.hi, O.scale.lo});
     if (O.flags & 1) z = ff_mul(z, FF{alpha.hi, alpha.lo});
     o[u] = z.hi + z.lo;
   }
-  *reinterpret_cast<float4*>(v + ((int64_t)O.out * KQ + kq) * 4) = make_float4(o[0], o[1], o[2], o[3]);
+  store_w<W>(v + (int64_t)O.out * RP + k, o);
 }
 
 // ---------------------------------------------------------------- row chunks
@@ -99,8 +142,9 @@ __global__ void k_gsum_mr(const GsumOut* __restrict__ outs, int nouts, const F2*
 // most of the launch: their slots are laid out [row][nt][tq], so that the four lanes
 // tq of a row read 64 consecutive bytes, with the loads of two rows in flight, and
 // y is updated four right-hand sides at a time (168 registers at 384 threads: all
-// eight spilled 136 bytes).  Row chunks of n = 1000, leaf 64, 32 columns: 53 us
-// with four pairs, 84 us with six and neither, 51 us now; H^2, n = 4000: 160, 194, 146 us.
+// eight spilled 136 bytes).  H, n = 1000, leaf 64, 32 columns: row chunks 51 us with four
+// pairs, 84 us with six and none of this, 40 us now; H^2, n = 4000, whole panel: 157, 178,
+// 117 us.
 constexpr int NT = RP / 8;
 constexpr int MP_NS = 2;                                   // stages per pair
 constexpr int MP_TP = RP * 4 + 16;                         // multiplier row pitch in a stage (bytes)
@@ -688,17 +732,24 @@ cudaError_t mr_init() {
   return e;
 }
 
+// Blocks of 256 threads for `items` entries of RP right-hand sides, W per thread.
+static unsigned blocks_w(int64_t items, int W) { return (unsigned)((items * (RP / W) + 255) / 256); }
+static bool fills(int64_t items) { return items * (RP / 4) >= MR_FULL; }
+
 cudaError_t launch_gather_mr(const double* x, int64_t ldx, int r, const int32_t* perm, int n, float* v,
                              cudaStream_t st) {
   if (n <= 0) return cudaSuccess;
-  return launch_pdl(k_gather_mr, (unsigned)(((int64_t)n * KQ + 255) / 256), 256, 0, st, x, ldx, r, perm, n, v);
+  if (fills(n)) return launch_pdl(k_gather_mr<4>, blocks_w(n, 4), 256, 0, st, x, ldx, r, perm, n, v);
+  return launch_pdl(k_gather_mr<1>, blocks_w(n, 1), 256, 0, st, x, ldx, r, perm, n, v);
 }
 
-cudaError_t launch_gsum_mr(const GsumOut* outs, int nouts, const F2* pscale, const float* partial, F2 alpha, float* v,
-                           cudaStream_t st) {
+// nterms: partials of all sums
+cudaError_t launch_gsum_mr(const GsumOut* outs, int nouts, int64_t nterms, const F2* pscale, const float* partial,
+                           F2 alpha, float* v, cudaStream_t st) {
   if (nouts <= 0) return cudaSuccess;
-  return launch_pdl(k_gsum_mr, (unsigned)(((int64_t)nouts * KQ + 255) / 256), 256, 0, st, outs, nouts, pscale, partial,
-                    alpha, v);
+  if (fills(nouts) && nterms <= MR_LONG * (int64_t)nouts)
+    return launch_pdl(k_gsum_mr<4>, blocks_w(nouts, 4), 256, 0, st, outs, nouts, pscale, partial, alpha, v);
+  return launch_pdl(k_gsum_mr<1>, blocks_w(nouts, 1), 256, 0, st, outs, nouts, pscale, partial, alpha, v);
 }
 
 // nblk ranges, one per warp

@@ -1101,6 +1101,7 @@ void finish_launches(Ctx& cx) {
         for (int64_t i = L.off; i < L.off + L.n; ++i) {
           const GsumOut& o = P.gouts[i];
           b += (int64_t)(o.p1 - o.p0) * ((o.flags & 2) ? 16 : 8) + (int64_t)sizeof(GsumOut) + 8;
+          L.nterms += o.p1 - o.p0;
         }
         break;
       case Launch::RGEMV:

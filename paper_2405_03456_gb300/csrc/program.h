@@ -69,6 +69,7 @@ struct Launch {
   int nw[NSHAPES] = {};           // ranges (warps; blocks for the multi-RHS shape) per launch shape
   int cfg = 0;                    // launch shape in use (autotuner choice)
   int maxrows = 0;                // RGEMV: rows of its widest chunk
+  int64_t nterms = 0;             // GSUM: partials of all its sums
   bool scatter = false;           // GSUM: also fills the slots of the folded fan-out after it
   int64_t copy_off = 0, copy_n = 0;  // GSUM with scatter: its copy entries fan_copy_{src,dst}[copy_off ..)
   int64_t xbytes = 0;             // bytes of that scatter (slot lists read, slots written)

@@ -102,7 +102,7 @@ LAUNCH(launch_prog, int, int, const ProgPhase*, int, const double*, const ItemCo
 LAUNCH(launch_cdot_tc, const ItemCopy*, I, int, const uint8_t*, const float*, F2, float*, float*, int*, S)
 LAUNCH(launch_cdot_ws, const ItemCopy*, I, int, const uint8_t*, const float*, F2, float*, float*, int*, S)
 LAUNCH(launch_gather_mr, const double*, int64_t, int, I, int, float*, S)
-LAUNCH(launch_gsum_mr, const GsumOut*, int, const F2*, const float*, F2, float*, S)
+LAUNCH(launch_gsum_mr, const GsumOut*, int, int64_t, const F2*, const float*, F2, float*, S)
 LAUNCH(launch_rgemv_tc, int, const PieceCopy*, I, int, const uint8_t*, const float*, double, F2, double, double*, int64_t,
        int, I, float*, const F2*, F2*, int32_t*, const Split*, I, int32_t, int*, S)
 LAUNCH(launch_rgemv_ms, int, const PieceCopy*, I, int, const uint8_t*, const float*, double, F2, double, double*, int64_t,

@@ -36,6 +36,20 @@ struct F2 {
   float hi, lo;
 };
 
+// A panel's row chunks are cut into ranges of pieces, a chunk that several ranges
+// share into parts (part k in the k-th range from the chunk's first one: no range of
+// a panel launch is empty).  The tensor-core kernel gives a CTA `per` consecutive
+// ranges, and the parts that fall to one CTA are one: what it does at the end of the
+// part in range `range` (its number `part` of `nparts`), with r1 the end of its ranges.
+struct CtaPart {
+  bool more;         // the chunk goes on in the CTA's next range: not an end
+  int idx, nparts;   // else number and count of the chunk's parts by CTA
+};
+HM_HD inline CtaPart cta_part(int range, int part, int nparts, int per, int r1) {
+  const int first = range - part, last = first + nparts - 1;   // ranges of the chunk
+  return CtaPart{range < last && range + 1 < r1, range / per - first / per, last / per - first / per + 1};
+}
+
 // First component of entry i in a vector that interleaves VS right-hand sides: a
 // program may have up to 2^31 entries, so that i * VS needs 64 bits.
 template <int VS>

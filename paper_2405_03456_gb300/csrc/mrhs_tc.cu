@@ -2,7 +2,8 @@
 // FP32 tier): y (or a coefficient panel) := the chunk rows of A times the
 // multiplier panel T, for panels of RP right-hand sides.
 //
-// One CTA owns a run of consecutive ranges of pieces (about MP_PAIRS, fewer where the launch is short); its warps have fixed roles and hand work on
+// One CTA owns a run of consecutive ranges of pieces (about MP_PAIRS, fewer where the
+// launch is short) as one stream; its warps have fixed roles and hand work on
 // through mbarriers (no block-wide barrier in the loop):
 //  * warp 0 streams every piece (one bulk copy) and its multiplier rows (RP
 //    values each, taken from the coefficient they stand for; 16-byte cp.async)
@@ -149,9 +150,10 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
   __shared__ uint32_t tbase;
   __shared__ int s_last;
   const int t = threadIdx.x, w = t >> 5, lane = t & 31;
-  // the CTA takes nrange / gridDim consecutive ranges as one stream of pieces (the
-  // ranges' part flags still hold: a chunk part closed at a range end goes
-  // through its fix-up slot like any other)
+  // the CTA takes nrange / gridDim consecutive ranges as one stream of pieces, and a
+  // chunk's parts in them as one part (cta_part): closing a part in each range, as the
+  // FP32-pipe kernel must, made panels of 128-row leaves slower with more ranges an SM
+  // (H, n = 2000, 32 columns: 109 us with four, 125 us with six, 54 us now)
   const int per = (nrange + (int)gridDim.x - 1) / (int)gridDim.x;
   const int r0 = blockIdx.x * per, r1 = min(r0 + per, nrange);
   if (r0 >= nrange) return;
@@ -373,8 +375,11 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
       fhi[e] = make_float2(0.f, 0.f);
       flo[e] = make_float2(0.f, 0.f);
     }
+    int range = r0, rend = wbeg[r0 + 1] - p0;   // of the piece, and where it ends
+    bool more = false;                          // the last piece's part goes on in this one
     for (int i = 0; i < n; ++i) {
       const int b = i & 1;
+      if (i == rend) rend = wbeg[++range + 1] - p0;   // (no range is empty)
       // the fold warps agree (they share a named barrier when they emit)
       const bool ok = mbar_wait(&dfull[b], (uint32_t)((i >> 1) & 1));
       int anybad;
@@ -389,7 +394,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
       }
       tc_fence_after();
       const TcInfo pi = dinfo[b];
-      if (pi.pd & PD_FIRST) {
+      if ((pi.pd & PD_FIRST) && !more) {
 #pragma unroll
         for (int e = 0; e < 8; ++e) {
           fhi[e] = make_float2(0.f, 0.f);
@@ -410,14 +415,20 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(&dempty[b]);
-      if (pi.pd & PD_LAST) {
+      Split sp{0, 1};
+      CtaPart cp{false, 0, 1};
+      if ((pi.pd & PD_LAST) && (pi.pd & PD_SPLIT)) {
+        sp = splits[pi.sp >> 8];
+        cp = cta_part(range, pi.sp & 0xff, sp.nparts, per, r1);
+      }
+      more = (pi.pd & PD_LAST) ? cp.more : false;
+      if ((pi.pd & PD_LAST) && !more) {
         const int R = pi.R;
         const bool calpha = (pi.flags & PH_CALPHA) != 0;
-        const bool split = (pi.pd & PD_SPLIT) != 0;
-        const Split sp = split ? splits[pi.sp >> 8] : Split{0, 1};
+        const bool split = cp.nparts > 1;
         bool emit = !split;
         if (split) {   // this part's rows, then the last part to arrive adds them all in part order
-          F2* mine = fix + (size_t)(sp.slot0 + (pi.sp & 0xff)) * CHUNK_ROWS * RP;
+          F2* mine = fix + (size_t)(sp.slot0 + cp.idx) * CHUNK_ROWS * RP;
           if (row < R) {
 #pragma unroll
             for (int e = 0; e < 8; ++e)
@@ -425,7 +436,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                   make_float4(fhi[e].x, flo[e].x, fhi[e].y, flo[e].y);
           }
           asm volatile("bar.sync 1, %0;" ::"r"(32 * TC_NEPI) : "memory");   // the fold warps' rows
-          if (te == 0) s_last = atom_add_acq_rel(&fixcnt[pi.sp >> 8], 1) == sp.nparts - 1;
+          if (te == 0) s_last = atom_add_acq_rel(&fixcnt[pi.sp >> 8], 1) == cp.nparts - 1;
           asm volatile("bar.sync 1, %0;" ::"r"(32 * TC_NEPI) : "memory");   // the acquire before the parts are read
           emit = s_last != 0;
           if (emit) {
@@ -434,7 +445,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
               fhi[e] = make_float2(0.f, 0.f);
               flo[e] = make_float2(0.f, 0.f);
             }
-            for (int part = 0; part < sp.nparts; ++part) {
+            for (int part = 0; part < cp.nparts; ++part) {
               const F2* src = fix + (size_t)(sp.slot0 + part) * CHUNK_ROWS * RP;
               if (row < R) {
 #pragma unroll

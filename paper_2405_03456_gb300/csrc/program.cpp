@@ -469,6 +469,10 @@ void add_rgemv(Ctx& cx, std::vector<ChunkWork>& cw, int mode, bool rowscale) {
       continue;
     }
     L.nw[cf] = partition(pb, L.off, cx.nsm * (cf == MR_SHAPE ? MP_PAIRS : RS_CFG_WARPS[cf]), P.wbeg);
+    if (cf == MR_SHAPE) {   // without the empty ranges (a piece above a range's share): cta_part counts on it
+      P.wbeg.erase(std::unique(P.wbeg.begin() + L.woff[cf], P.wbeg.end()), P.wbeg.end());
+      L.nw[cf] = (int)((int64_t)P.wbeg.size() - L.woff[cf]) - 1;
+    }
     std::vector<PieceCopy> d = base;
     std::vector<int32_t> nparts(cw.size(), 0), partof(pw.size(), 0);
     const int32_t* wb = P.wbeg.data() + L.woff[cf];

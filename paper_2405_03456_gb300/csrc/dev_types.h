@@ -310,6 +310,22 @@ struct LuCItem {                 // a column item: columns [c0, c0 + nc), nc <= 
   int32_t bwd;
 };
 
+// Bound of a wait for a number that others advance (the solve's frontier): it gives up
+// when `limit` tries in a row saw no progress, however long the whole wait is.
+struct Patience {
+  uint32_t limit, left;
+  int last;
+  HM_HD explicit Patience(uint32_t n) : limit(n), left(n), last(-1) {}
+  // After a try that read v and has to go on: whether another one may follow.
+  HM_HD bool again(int v) {
+    if (v != last) {
+      last = v;
+      left = limit;
+    }
+    return --left > 0;
+  }
+};
+
 enum { MODE_Y = 0, MODE_VEC = 1, MODE_VEC_ADD = 2 };
 enum { TIER_F32 = 0, TIER_FF = 1 };
 

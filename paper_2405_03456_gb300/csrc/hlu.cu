@@ -37,8 +37,9 @@
 // A step or item waits only for earlier ones in the work list, both kinds are
 // claimed in list order and all blocks are resident: the earliest unfinished one
 // never waits for anything unfinished, so the launch cannot stall.  Every wait is
-// bounded; after the first that runs out the abort word makes all later ones
-// return at once, and the launch runs to its end.
+// bounded by the time without a finished step (Patience), so that neither a long
+// solve nor a GPU shared with other work runs into it; after the first that runs out
+// the abort word makes all later ones return at once, and the launch runs to its end.
 #include <cstdint>
 #include <cuda_runtime.h>
 
@@ -95,12 +96,14 @@ __device__ __forceinline__ void lu_fail(const LuArgs& A) {
   latch_error(A.err, 99);
 }
 
-// Wait (bounded, about 2 s) until `need` steps are finished.
+// Wait until `need` steps are finished (bounded: about 2 s without a step).
 template <int NR>
 __device__ __forceinline__ void wait_front(const LuArgs& A, uint32_t sf, int need) {
-  for (uint32_t i = 0; i < (1u << 26); ++i) {
+  Patience p(1u << 26);
+  for (;;) {
     const int v = front_load(sf);
     if (v >= need * NR || v < 0) return;
+    if (!p.again(v)) break;
   }
   lu_fail(A);
 }
@@ -110,9 +113,13 @@ template <int NR>
 __device__ __forceinline__ void wait_col(const LuArgs& A, uint32_t sf, const LuSCol& c) {
   wait_front<NR>(A, sf, c.need);
   if (c.flag < 0) return;
-  for (uint32_t i = 0; i < (1u << 22); ++i) {   // each try is an L2 round trip: about 2 s in all
-    if (ld_acquire(A.flags + c.flag) >= c.target) return;
-    if ((i & 63u) == 63u && front_load(sf) < 0) return;
+  Patience p(1u << 16);
+  for (;;) {   // 64 tries of an L2 round trip each, then a look at the frontier: about 2 s without a step
+    for (int i = 0; i < 64; ++i)
+      if (ld_acquire(A.flags + c.flag) >= c.target) return;
+    const int v = front_load(sf);
+    if (v < 0) return;
+    if (!p.again(v)) break;
   }
   lu_fail(A);
 }
@@ -429,12 +436,14 @@ __global__ void __launch_bounds__(LU_THREADS, 1) k_lusolve(LuArgs A, int row_blo
     if (lane == 0) {
       const int total = A.nsteps * NR;
       int v = 0;
-      for (uint32_t i = 0; i < (1u << 24) && v < total; ++i) {
+      Patience p(1u << 24);
+      for (uint32_t i = 0; v < total; ++i) {
         v = ld_acquire(A.frontier);
         if ((i & 31u) == 31u && *(volatile int*)A.abort) break;
         front_store(sf, v);
+        if (!p.again(v)) break;
       }
-      if (v < total) {   // an abort, or no progress for seconds
+      if (v < total) {   // an abort, or no step for seconds
         lu_fail(A);
         front_store(sf, -1);
       }

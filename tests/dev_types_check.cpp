@@ -23,7 +23,21 @@ static void offsets() {
     if (i <= std::numeric_limits<int32_t>::max()) CHECK(entry_offset<VS>((int32_t)i) == i * VS);
 }
 
+// Tries until a wait on `value(try)` gives up, at most `max`.
+template <class F>
+static int64_t tries(uint32_t limit, int64_t max, F value) {
+  Patience p(limit);
+  int64_t i = 0;
+  while (i < max && p.again(value(i))) ++i;
+  return i;
+}
+
 int main() {
+  // a number that never moves: limit tries; one that moves within the limit: no end; one that stops: limit more
+  CHECK(tries(100, 10000, [](int64_t) { return 7; }) == 99);
+  CHECK(tries(100, 100000, [](int64_t i) { return (int)(i / 99); }) == 100000);
+  CHECK(tries(100, 100000, [](int64_t i) { return (int)(i < 5000 ? i / 50 : 99); }) == 4950 + 99);
+  CHECK(tries(100, 10000, [](int64_t) { return 0; }) == 99);
   offsets<1>();
   offsets<2>();
   offsets<4>();

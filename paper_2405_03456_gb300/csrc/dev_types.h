@@ -310,6 +310,12 @@ struct LuCItem {                 // a column item: columns [c0, c0 + nc), nc <= 
   int32_t bwd;
 };
 
+// Steps that must be finished before every row of a 64-row piece of a column item is
+// final, given the leaf indices of its first and last row (nl leaves).
+HM_HD inline int lu_piece_need(bool fwd, int nl, int leaf_first, int leaf_last) {
+  return fwd ? leaf_last + 1 : 2 * nl - leaf_first;
+}
+
 // Bound of a wait for a number that others advance (the solve's frontier): it gives up
 // when `limit` tries in a row saw no progress, however long the whole wait is.
 struct Patience {

@@ -392,7 +392,7 @@ __device__ void lu_citem(const LuArgs& A, int ci, uint32_t sf, int lane) {
   auto fetch = [&](int p) {   // codes and the required step of piece p
     const int a = 64 * p, b = min(it.nr, a + 64);
     if (on && a + RPL * q < it.nr) lu_raw(A, c, 8 * p + q, raw);
-    need = fwd ? __ldg(A.rowleaf + it.r0 + b - 1) + 1 : 2 * A.nl - __ldg(A.rowleaf + it.r0 + a);
+    need = lu_piece_need(fwd, A.nl, __ldg(A.rowleaf + it.r0 + a), __ldg(A.rowleaf + it.r0 + b - 1));
   };
   fetch(fwd ? 0 : np - 1);
   for (int k = 0; k < np; ++k) {

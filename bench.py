@@ -256,7 +256,7 @@ def profiled_traffic(kernel, n):
         rec = dict(ln.split(" ", 1) for ln in open(os.path.join(ROOT, "profiles", "k_rstream_traffic.txt")).read()
                    .strip().splitlines())
         src = b"".join(open(os.path.join(ROOT, "paper_2405_03456_gb300", "csrc", f), "rb").read()
-                       for f in ("kernels.cu", "decode.cuh", "dev_types.h"))
+                       for f in ("kernels.cu", "stream.cuh", "decode.cuh", "dev_types.h"))
     except OSError:
         return None
     if rec.get("kernel") != kernel or f"N={n} " not in rec.get("workload", ""):
@@ -613,7 +613,8 @@ def gpu_arm(args, rank, world):
         "by_eps": by_eps,
         "by_nrhs": {"workload": "the headline matrix, Y := M X with r right-hand sides (panels of 32 on the "
                                "multi-RHS engine the autotuner chose: FP32 pipes, or tcgen05 tensor cores with exact "
-                               "BF16 limbs; per-piece FP32 sums, float-float across pieces; r < 9 as single products)",
+                               "BF16 limbs; per-piece FP32 sums, float-float across pieces; "
+                               "r < 9 as batches of 2, 4 or 8 columns, one column as a single product)",
                     "engine": headline.get("multi_rhs_engine"),
                     **headline.get("by_nrhs", {})},
         "by_format": {f"{f}-{c}": {"gbs": round(r["gbs"], 1), "ms_p50": round(r["ms_p50"], 4),

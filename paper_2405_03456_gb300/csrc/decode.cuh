@@ -353,17 +353,15 @@ __device__ __forceinline__ void ff_add_dot2(float2& hi, float2& lo, float2 s, fl
 // 8 consecutive codes of format (F, B) at shared address a -> 4 FP32 pairs
 // (FP32 tier: AFLP as +-(s - 1), FPX e8 exactly, e11 / raw cut to FP32; see
 // decode4 for what each class gives).
-template <int B>
-__device__ __forceinline__ void load8(uint32_t a, uint32_t (&w)[2 * B]) {
+template <int F, int B>
+__device__ __forceinline__ void decode8p(uint32_t a, int e, int m, float2 (&h2)[4]) {
+  uint32_t w[2 * B];
 #pragma unroll
   for (int i = 0; i < B; ++i) {
     const uint2 t = lds64(a + 8u * i);
     w[2 * i] = t.x;
     w[2 * i + 1] = t.y;
   }
-}
-template <int F, int B>
-__device__ __forceinline__ void decode8w(const uint32_t (&w)[2 * B], int e, int m, float2 (&h2)[4]) {
   uint32_t w0[B], w1[B];
 #pragma unroll
   for (int i = 0; i < B; ++i) {
@@ -402,13 +400,6 @@ __device__ __forceinline__ void decode8w(const uint32_t (&w)[2 * B], int e, int 
     h2[2] = make_float2(h1[0], h1[1]);
     h2[3] = make_float2(h1[2], h1[3]);
   }
-}
-
-template <int F, int B>
-__device__ __forceinline__ void decode8p(uint32_t a, int e, int m, float2 (&h2)[4]) {
-  uint32_t w[2 * B];
-  load8<B>(a, w);
-  decode8w<F, B>(w, e, m, h2);
 }
 
 // ---------------------------------------------------------------- tensor-core helpers

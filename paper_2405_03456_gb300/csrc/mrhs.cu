@@ -17,8 +17,6 @@
 
 namespace hm {
 
-__device__ __forceinline__ uint32_t pad16m(uint32_t x) { return (x + 15u) & ~15u; }
-
 // ---------------------------------------------------------------- gather, segment sums
 // W right-hand sides per thread.  W = 4 (independent loads, one 16-byte store) has more
 // loads in flight where its threads alone fill the GPU (MR_FULL) and the sums are
@@ -310,7 +308,7 @@ __global__ void __launch_bounds__(MP_THREADS, 1)
     const int32_t sp = __shfl_sync(HM_FULL, dc.split_part, sl);
     const int s = i % MP_NS;
     uint8_t* st = ring + (size_t)s * MP_STAGE;
-    const uint32_t nc = bf >> 24, pb = pad16m(bf & 0xffffu);
+    const uint32_t nc = bf >> 24, pb = pad16u(bf & 0xffffu);
     fence_proxy_async();
     if (lane == 0) {
       info[pair][s] = make_int4((int)((bf >> 16) & 0xffu), sp, 0, 0);
@@ -616,7 +614,7 @@ __device__ __forceinline__ void cw_piece(uint32_t sa, uint32_t scr, int R, int n
         partial[o] = tot;
       }
     };
-    if (j0 + 4 <= nc) {   // in pairs: independent reductions
+    if (j0 + 4 <= nc) {   // independent reductions
       column(0);
       column(1);
       column(2);
@@ -658,7 +656,7 @@ __global__ void __launch_bounds__(CW_WARPS * 32, 1)
     const uint32_t off16 = __shfl_sync(HM_FULL, dc.off16, sl), bytes = __shfl_sync(HM_FULL, dc.bytes, sl);
     if (lane == 0) {
       const int s = i % CW_NS;
-      const uint32_t pb = pad16m(bytes);
+      const uint32_t pb = pad16u(bytes);
       fence_proxy_async();
       mbar_expect_tx(&bars[s], pb);
       bulk_g2s_hint(ring + (size_t)s * STAGE_BYTES, pay + (uint64_t)off16 * 16u, pb, &bars[s], pol);

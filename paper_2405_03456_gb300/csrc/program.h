@@ -137,7 +137,7 @@ struct LuProgram {
   Packer pk;
   std::vector<LuCol> cols;
   std::vector<LuItem> items;
-  std::vector<LuDep> deps;
+  std::vector<LuDep> deps;  // of the list's items, for its replay on the host; the device waits by the steps of schedule_lu
   int64_t nflags = 0;       // done flags (2 per leaf) and coefficient counters
   int64_t ncoef = 0;        // coefficients of the low-rank blocks of both factors
   int64_t nleaves = 0;

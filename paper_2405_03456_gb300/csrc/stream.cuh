@@ -30,7 +30,8 @@ __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;"
 // Range of warp (or pair) w of this block.  A launch with fewer ranges than warps
 // on the device gets one block per SM all the same and deals its ranges out over
 // the blocks, so that a short launch uses every SM (16 ranges on one SM share its
-// issue slots while others idle); a full one keeps neighbouring ranges together.
+// issue slots while others idle).  So does a launch whose last block is not full; one
+// whose ranges fill its blocks exactly keeps neighbouring ranges together.
 template <int NW>
 __device__ __forceinline__ int range_of(int w, int nranges) {
   return (int)gridDim.x * NW > nranges ? w * (int)gridDim.x + (int)blockIdx.x : (int)blockIdx.x * NW + w;

@@ -113,12 +113,10 @@ hm_status hm_compress(hm_matrix* m, double eps, int32_t codec, int32_t valr);
  *   y : device, FP64, n x nrhs, leading dimension ldy >= n; must not overlap x.
  *   nrhs : 1..64 right-hand sides.  FP32 tier: panels of up to 32 columns while 9 or
  *     more are left; what remains, and every column of the float-float tier, in
- *     batches of 2, 4 or 8 (float-float: 2 or 4) and single products (one column,
- *     the fifth of five, two columns of a matrix whose row-chunk launches are fused
- *     into runs, H^2 and separate couplings; and all of them when the device had no
- *     room for the batch buffers at hm_compress).  A panel or a batch reads the matrix
- *     once; a batch column equals its single product up to the float-float order of
- *     summation across pieces.
+ *     batches of 2, 4 or 8 (float-float: 2 or 4) and single products (one column, the
+ *     fifth of five; all of them when the device had no room for the batch buffers at
+ *     hm_compress).  A panel or a batch reads the matrix once; a batch column equals
+ *     its single product up to the float-float order of summation across pieces.
  *   stream : cudaStream_t as void* (NULL = default stream).
  * Concurrent calls on one matrix must be ordered by the caller (they share the
  * matrix's workspace).  Device-side errors are latched, see hm_sync_status.

@@ -757,7 +757,9 @@ static hm_status run_program_b(hm_matrix* M, int nv, double alpha, const double*
 // FP32 tier, N = 131072, eps = 1e-6 (ms): 1 column 0.222, 2 0.364, 3 0.465 and 4
 // 0.478 (width 4), 6 .. 8 0.85 (width 8), 5 0.70 as 4 + 1 and 0.79 at width 8; before,
 // 0.22 a column.  Float-float, n = 32768, eps = 1e-8: 0.159, 0.281, 0.476 at width 4;
-// before, 0.174 a column.
+// before, 0.174 a column.  Also where a single product's row-chunk launches are fused
+// into runs and a batch's are not: two columns as a batch / as two single products, us,
+// H^2 n = 2048 68 / 100, n = 32768 222 / 261; UH separate n = 2048 43 / 80, n = 16384 82 / 126.
 static int pass_width(int tier, int64_t rem) {
   if (rem <= 1) return 1;
   if (rem == 2) return 2;
@@ -767,7 +769,9 @@ static int pass_width(int tier, int64_t rem) {
 // All right-hand sides: panels of RP through the multi-RHS kernels (FP32
 // tier), the rest (or everything in the float-float tier) in batch passes.  A
 // panel reads the matrix once, but costs more than a batch pass, so remainders
-// below MR_MIN_RHS run as batches.
+// below MR_MIN_RHS run as batches (H n = 32768, us: 8 columns 209 as a batch, a panel
+// 306 whatever its columns; N = 131072: 0.83 and 1.36 ms).  The best line depends on
+// the matrix: H^2 n = 32768 takes 8 columns in 706 us as a batch, 370 as a panel.
 constexpr int64_t MR_MIN_RHS = 9;
 static hm_status run_all(hm_matrix* M, double alpha, const double* x, int64_t ldx, double beta, double* y,
                          int64_t ldy, int64_t nrhs, cudaStream_t st) {
@@ -778,10 +782,7 @@ static hm_status run_all(hm_matrix* M, double alpha, const double* x, int64_t ld
       s = run_program_mr(M, alpha, x + r0 * ldx, ldx, beta, y + r0 * ldy, ldy, (int)std::min<int64_t>(RP, nrhs - r0),
                          st);
   while (r0 < nrhs && s == HM_OK) {
-    // two columns of a matrix with fused runs (H^2, UH separate) are not slower as
-    // single products: their launches are short, and a batch runs them one by one
-    const bool single = !M->d_vb || (nrhs - r0 <= 2 && M->fuse && !M->runs.empty());
-    const int nv = single ? 1 : pass_width(M->prog.tier, nrhs - r0);
+    const int nv = M->d_vb ? pass_width(M->prog.tier, nrhs - r0) : 1;
     const int r = (int)std::min<int64_t>(nv, nrhs - r0);
     if (nv == 1)
       s = run_program(M, alpha, x + r0 * ldx, beta, y + r0 * ldy, st);

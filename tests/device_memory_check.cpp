@@ -6,7 +6,8 @@
 // are optional: once a budget suffices, no larger one may fail, the smallest that
 // suffices runs single products and the largest runs batches.  Everything allocated
 // is freed.
-// usage: device_memory_check <points file> n eps codec leaf
+// Two to eight right-hand sides run as batches in every format when the buffers are there.
+// usage: device_memory_check <points file> n eps codec leaf format
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
@@ -120,7 +121,7 @@ int batch_shape(int, int) { return 1; }
 }  // namespace hm
 
 int main(int argc, char** argv) {
-  if (argc != 6) return 2;
+  if (argc != 7) return 2;
   const int64_t n = std::atoll(argv[2]);
   std::vector<double> pts(3 * n), x(64 * n, 1.0), y(64 * n, 0.0);
   FILE* f = std::fopen(argv[1], "rb");
@@ -131,6 +132,7 @@ int main(int argc, char** argv) {
   prm.eta = 2.0;
   prm.eps_build = std::atof(argv[3]);
   prm.leaf_size = std::atoi(argv[5]);
+  prm.format = std::atoi(argv[6]);
   prm.nthreads = 4;
   struct Result {
     hm_status s;
@@ -153,6 +155,15 @@ int main(int argc, char** argv) {
     CHECK(g_used == 0 && g_mem.empty());
     return r;
   };
+  g_budget = size_t(1) << 40;
+  for (int r = 2; r <= 8; ++r) {
+    hm_matrix* M = nullptr;
+    CHECK(hm_build(&prm, pts.data(), n, &M) == HM_OK && hm_compress(M, prm.eps_build, std::atoi(argv[4]), 1) == HM_OK);
+    g_calls.clear();
+    CHECK(hm_matvec(M, 1.0, x.data(), n, 0.0, y.data(), n, r, nullptr) == HM_OK);
+    CHECK(g_calls["launch_gather_b"] >= 1 && g_calls["launch_gather"] <= (r == 5));
+    hm_free(M);
+  }
   const Result all = attempt(size_t(1) << 40);
   CHECK(all.s == HM_OK && all.batch);
   // budgets up to that use and the room that batches ask for, in steps finer than any of their buffers' sum

@@ -28,12 +28,13 @@ def checker(tmp_path_factory):
     return exe, tmp
 
 
-@pytest.mark.parametrize("n,eps,codec,leaf", [(1500, "1e-8", 1, 32), (700, "1e-4", 0, 64), (1500, "1e-6", 1, 32),
-                                              (300, "1e-6", 2, 128)])
-def test_optional_buffers_never_cost_a_matrix(checker, n, eps, codec, leaf):
+@pytest.mark.parametrize("n,eps,codec,leaf,fmt", [(1500, "1e-8", 1, 32, 0), (400, "1e-4", 0, 64, 0),
+                                                  (1500, "1e-6", 1, 32, 0), (300, "1e-6", 2, 128, 0),
+                                                  (1200, "1e-6", 1, 64, 2), (700, "1e-6", 1, 32, 3)])
+def test_optional_buffers_never_cost_a_matrix(checker, n, eps, codec, leaf, fmt):
     exe, tmp = checker
     path = tmp / f"sphere_{n}.bin"
     path.write_bytes(np.ascontiguousarray(synth.sphere_points(n)).tobytes())
-    r = subprocess.run([exe, str(path), str(n), eps, str(codec), str(leaf)], stdout=subprocess.PIPE,
+    r = subprocess.run([exe, str(path), str(n), eps, str(codec), str(leaf), str(fmt)], stdout=subprocess.PIPE,
                        stderr=subprocess.STDOUT, text=True, timeout=600)
     assert r.returncode == 0 and r.stdout.rstrip().endswith("ok"), r.stdout[-2000:]

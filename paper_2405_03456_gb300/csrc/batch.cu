@@ -18,8 +18,9 @@
 //    coefficients (source indices one piece ahead), so a batch needs no fan-out;
 //  * fewer, fatter warps than the single kernels: the NV independent sums of a
 //    lane hide the latency that 16 warps per SM hide there.
-// Measured (AFLP): N = 131072, eps = 1e-6, 4 columns 0.475 ms, 8 columns 0.83 ms (0.88
-// and 1.76 as single products); n = 32768, eps = 1e-8, 4 columns 0.48 ms (0.70).
+// Measured (AFLP): N = 131072, eps = 1e-6, 4 columns 0.473 ms, 8 columns 0.84 ms (0.88
+// and 1.76 as single products); n = 32768, eps = 1e-8, 4 columns 0.48 ms (0.70).  The
+// row chunks of 8 columns take all 255 registers of a thread (4 bytes spilled).
 #include <cstdint>
 #include <cuda_runtime.h>
 
@@ -112,7 +113,7 @@ __global__ void k_gsum_b(const GsumOut* __restrict__ outs, int nouts, const F2* 
 // decoder alone.  In the float-float tier the arithmetic of NV right-hand sides is
 // several times the decoder's code: it exists once (class F < 0 below), because
 // one copy for each class in use does not fit the instruction cache (NV = 4 column
-// dots, n = 32768, eps = 1e-8: 515 us with the copies, 244 us so).
+// dots, n = 32768, eps = 1e-8: 515 us with the copies, 233 us so).
 template <int TIER, int F, int B>
 __device__ __forceinline__ void decode_b(uint32_t fb, uint32_t a, int e, int m, float (&h)[8], float (&l)[8]) {
   if constexpr (F >= 0) {

@@ -771,7 +771,7 @@ static int pass_width(int tier, int64_t rem) {
 // panel reads the matrix once, but costs more than a batch pass, so remainders
 // below MR_MIN_RHS run as batches (H n = 32768, us: 8 columns 209 as a batch, a panel
 // 306 whatever its columns; N = 131072: 0.83 and 1.36 ms).  The best line depends on
-// the matrix: H^2 n = 32768 takes 8 columns in 706 us as a batch, 370 as a panel.
+// the matrix: H^2 n = 32768 takes 8 columns in 708 us as a batch, 380 as a panel.
 constexpr int64_t MR_MIN_RHS = 9;
 static hm_status run_all(hm_matrix* M, double alpha, const double* x, int64_t ldx, double beta, double* y,
                          int64_t ldy, int64_t nrhs, cudaStream_t st) {
